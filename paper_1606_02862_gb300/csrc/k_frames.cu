@@ -12,6 +12,8 @@
 //     the kept frame indices, pops new frames off the free stack and queues
 //     released ones;
 //   place: every waiting particle goes to slot abase[L] + rank of its list;
+//     the same launch lists the supercells that hold mobile particles for
+//     the next push;
 //   free_push: released frames go back on the free stack.
 // Loading particles from the host uses the same path: a conversion kernel
 // fills the move buffer, then the maintenance places them.
@@ -129,6 +131,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const StepDev d)
 {
     const int4 tot = *d.totals;
     const int top = *d.free_top;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *d.nitems = 0;  // k_place counts them anew
     if (tot.y > top) {
         // pool exhausted: report it; the step's arrivals are abandoned
         if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -170,11 +174,50 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const StepDev d)
     }
 }
 
-__global__ void k_place(const StepDev d)
+// The work items of the next push: the supercells with a particle of a
+// mobile species, 32 at a time (one ballot and one atomic per warp that has
+// any; *d.nitems starts at zero).  In a mostly empty box the push otherwise
+// spends its time asking for supercells that it then skips: a 256^3 box
+// without particles took 0.395 ms per push (131,072 skipped items), of a
+// step of 0.83 ms.
+__device__ __forceinline__ void list_items(const StepDev& d)
+{
+    const int lane = threadIdx.x & 31;
+    for (int b = (int)(blockIdx.x * blockDim.x + threadIdx.x) - lane; b < d.nsc; b += (int)(gridDim.x * blockDim.x)) {
+        const int g = b + lane;
+        bool any = false;
+        if (g < d.nsc)
+            for (int s = 0; s < d.nspecies; ++s)
+                any = any || (d.sp[s].mobile && d.count[s * d.nsc + g] > 0);
+        const unsigned m = __ballot_sync(0xffffffffu, any);
+        if (m == 0)
+            continue;
+        int base = 0;
+        if (lane == 0)
+            base = atomicAdd(d.nitems, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (any)
+            d.items[base + __popc(m & ((1u << lane) - 1u))] = g;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_list_items(const StepDev d) { list_items(d); }
+
+cudaError_t launch_list_items(const StepDev& d, int blocks, cudaStream_t st)
+{
+    const cudaError_t e = cudaMemsetAsync(d.nitems, 0, sizeof(int), st);
+    if (e != cudaSuccess)
+        return e;
+    k_list_items<<<blocks, 256, 0, st>>>(d);
+    return cudaGetLastError();
+}
+
+__global__ void __launch_bounds__(256) k_place(const StepDev d)
 {
     const int4 tot = *d.totals;
     if (tot.y > *d.free_top)
         return;
+    list_items(d);
     const int n = min(*d.mv_count, d.mv_cap);
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
         const int L = d.mv_dest[m];

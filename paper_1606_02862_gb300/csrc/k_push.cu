@@ -3,7 +3,8 @@
 //
 // One CTA works on one supercell at a time (Sec. 2.1: a supercell maps to a
 // block, its threads share the supercell's particles); CTAs are persistent
-// and pull supercells from a work counter (one item ahead), so boxes of any
+// and pull the supercells that hold mobile particles (a list that the frame
+// maintenance writes) from a work counter, one item ahead, so boxes of any
 // size and occupancy share one launch.  Per supercell:
 //   1. stage the E and B tile (supercell + G guard cells below, G = 1 for
 //      CIC/TSC, 2 with PCS) from HBM into shared memory with 16-byte
@@ -649,7 +650,7 @@ struct SharedState {
     int off[max_keys<T>()];
     unsigned long long mb_tile;    // completion of the E/B tile's tensor loads
     unsigned alive[NQ * NT / 32];  // per warp and pass: ballot of the pushed particles that stay
-    int item, any, nlv, lv_base;
+    int item, nlv, lv_base;
     int tile_phase;                // parity of the tile barrier's next phase
     int abort;                     // the tile wait gave up
     int ngen[2];             // general-window moves of the chunk
@@ -1433,9 +1434,10 @@ __global__ void __launch_bounds__(NT, (T::G == 1 ? 1024 : 512) / NT) k_push_depo
     if (T::G == 2 && tid < 32)
         sh.bh[tid] = 0;  // each chunk clears it after use
     __syncthreads();
+    const int nitems = *d.nitems;
     for (;;) {
         const int item = sh.item;
-        if (item >= d.nsc)
+        if (item >= nitems)
             break;
         int next_item = 0;
         if (tid == 0)
@@ -1450,24 +1452,8 @@ __global__ void __launch_bounds__(NT, (T::G == 1 ? 1024 : 512) / NT) k_push_depo
         const int scy = (loc / bx.nscx) % bx.nscy;
         const int scz = loc / (bx.nscx * bx.nscy);
 
-        if (tid == 0) {
-            int ntot = 0;
-            for (int s = 0; s < d.nspecies; ++s) {
-                const int c = d.count[s * d.nsc + g];
-                if (d.sp[s].mobile && c > 0)
-                    ntot += c;
-            }
-            sh.any = ntot;
+        if (tid == 0)
             sh.nlv = 0;  // every thread read it in flush_leavers (before its barrier, if it had one)
-        }
-        __syncthreads();
-        if (sh.any == 0) {
-            if (tid == 0)
-                sh.item = next_item;
-            __syncthreads();  // item / any are rewritten next round
-            continue;
-        }
-
 
         // ---- 1. the E/B tile by two tensor loads (TMA); on a stored-order
         // pass the first chunk of the first mobile list is copied meanwhile;
@@ -1489,7 +1475,7 @@ __global__ void __launch_bounds__(NT, (T::G == 1 ? 1024 : 512) / NT) k_push_depo
             const CUtensorMap* tm = d.tmaps + 2 * d.sc_box[g];
             tma_load_tile(sF, tm, scx * LX, scy * LY, scz * LZ, &sh.mb_tile);
             tma_load_tile(sF + T::BOFF, tm + 1, scx * LX, scy * LY, scz * LZ, &sh.mb_tile);
-            if (next_item < d.nsc) {
+            if (next_item < nitems) {
                 const int gn = d.items[next_item];
                 const int bn = d.sc_box[gn];
                 const BoxDev& bxn = d.boxes[bn];

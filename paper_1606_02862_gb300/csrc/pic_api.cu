@@ -76,7 +76,7 @@ struct pic_ctx {
     BoxDev* boxes_d = nullptr;
     CUtensorMap* tmaps_d = nullptr;  // [nboxes][2] E, B tile maps of the push
     int* sc_box_d = nullptr;
-    int* items_d = nullptr;
+    int* items_d = nullptr;   // [nsc] work items of the push, and after them their number
     int* yee_off_d = nullptr;
     int yee_nblocks = 0;
     float *E_all = nullptr, *B_all = nullptr, *J_all = nullptr;
@@ -389,6 +389,7 @@ StepDev make_step(const pic_ctx* c, int parity, bool alt = false)
     d.tmaps = alt ? c->tmaps_alt_d : c->tmaps_d;
     d.sc_box = c->sc_box_d;
     d.items = c->items_d;
+    d.nitems = c->items_d + c->nsc;
     const double V = c->h[0] * c->h[1] * c->h[2];
     for (size_t s = 0; s < c->sp.size(); ++s) {
         const pic_species& p = c->sp[s];
@@ -1294,12 +1295,9 @@ pic_status pic_create(const pic_grid* grids, int32_t nboxes, const double dx[3],
             for (int i = 0; i < bd.nscx * bd.nscy * bd.nscz; ++i)
                 sc_box[bd.sc_base + i] = b;
         }
-        std::vector<int> items(nsc);
-        for (int i = 0; i < nsc; ++i)
-            items[i] = i;
         const int nblk = (c->nlists + 4095) / 4096;
         if (dalloc(c, &c->boxes_d, nboxes, false) != PIC_OK || dalloc(c, &c->sc_box_d, nsc, false) != PIC_OK ||
-            dalloc(c, &c->items_d, nsc, false) != PIC_OK || dalloc(c, &c->yee_off_d, nboxes + 1, false) != PIC_OK ||
+            dalloc(c, &c->items_d, nsc + 1) != PIC_OK || dalloc(c, &c->yee_off_d, nboxes + 1, false) != PIC_OK ||
             dalloc(c, &c->count, c->nlists) != PIC_OK || dalloc(c, &c->nframes, c->nlists) != PIC_OK ||
             dalloc(c, &c->narrive, c->nlists) != PIC_OK || dalloc(c, &c->abase, c->nlists) != PIC_OK ||
             dalloc(c, &c->foff[0], c->nlists) != PIC_OK || dalloc(c, &c->foff[1], c->nlists) != PIC_OK ||
@@ -1312,8 +1310,6 @@ pic_status pic_create(const pic_grid* grids, int32_t nboxes, const double dx[3],
         if (cudaMemcpyAsync(c->boxes_d, c->boxes_h.data(), sizeof(BoxDev) * nboxes,
                             cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
             cudaMemcpyAsync(c->sc_box_d, sc_box.data(), sizeof(int) * nsc, cudaMemcpyHostToDevice,
-                            c->stream) != cudaSuccess ||
-            cudaMemcpyAsync(c->items_d, items.data(), sizeof(int) * nsc, cudaMemcpyHostToDevice,
                             c->stream) != cudaSuccess ||
             cudaMemcpyAsync(c->yee_off_d, yee_off.data(), sizeof(int) * (nboxes + 1),
                             cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
@@ -1444,6 +1440,7 @@ pic_status pic_shift_window(pic_ctx* c, int32_t box, int32_t cells)
                        cudaMemcpyDeviceToDevice, c->stream));
     d = make_step(c, c->parity);
     CK(launch_rotate_lists(d, b, c->rot_scratch, c->foff[c->parity], rows, c->stream));
+    CK(launch_list_items(d, 4 * c->nsm, c->stream));
     // a shift by whole supercells keeps every particle's cell and its list
     // order: nothing else to redo
     CK(cudaStreamSynchronize(c->stream));

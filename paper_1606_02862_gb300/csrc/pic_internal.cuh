@@ -94,7 +94,8 @@ struct StepDev {
     const BoxDev* boxes;      // [nboxes]
     const CUtensorMap* tmaps; // [nboxes][2]: the E and B tile loads of the push (TMA)
     const int* sc_box;        // [nsc] box of each global supercell
-    const int* items;         // [nsc] supercells in work order
+    int* items;               // [nsc] the supercells that hold mobile particles, in work order
+    int* nitems;              // device scalar: how many
     SpeciesDev sp[kMaxSpecies];
     // particle pool
     int* cell;
@@ -250,6 +251,8 @@ int absorber_blocks(const BoxDev& b);
 cudaError_t launch_shift_fields(const BoxDev& b, float* F, const float* scratch, int cells,
                                 cudaStream_t st);
 cudaError_t launch_clear_rows(const StepDev& d, const BoxDev& hb, int rows, cudaStream_t st);
+// rebuild d.items from the particle counts (launch_frame_apply does it too)
+cudaError_t launch_list_items(const StepDev& d, int blocks, cudaStream_t st);
 cudaError_t launch_rotate_lists(const StepDev& d, const BoxDev& hb, const int* old3, int* foff,
                                 int rows, cudaStream_t st);
 cudaError_t launch_fields_to_padded(const BoxDev& b, int which, const double* src,
