@@ -335,10 +335,28 @@ __device__ __forceinline__ float2 gather_pair(const float* __restrict__ F1, int 
     return acc;
 }
 
-// Esirkepov transverse factor S0e S0f + (DSe S0f + S0e DSf)/2 + DSe DSf / 3.
-__device__ __forceinline__ float esk_T(float s0e, float dse, float s0f, float dsf)
+// Esirkepov's transverse factor S0e S0f + (DSe S0f + S0e DSf)/2 + DSe DSf / 3
+// as A S0f + B DSf with A = S0e + DSe / 2, B = S0e / 2 + DSe / 3: A and B
+// belong to one node of axis e, so that a line of the window takes two
+// operations instead of seven (27 lines per TSC move; the TSC push of 256^3
+// cells at 8 particles each went from 9.97 to 9.73 ms).  CIC moves (12 lines
+// in the common window) keep the form of esk_T_cic and its rounding: the
+// energy-conserving CIC gather jumps at half a cell, where another rounding of
+// the current now and then gives a particle another kick.
+__device__ __forceinline__ float esk_A(float s0, float ds) { return fmaf(0.5f, ds, s0); }
+__device__ __forceinline__ float esk_B(float s0, float ds) { return fmaf(0.5f, s0, (1.0f / 3.0f) * ds); }
+
+__device__ __forceinline__ float esk_T_cic(float s0e, float dse, float s0f, float dsf)
 {
     return fmaf(s0e, s0f, fmaf(0.5f, fmaf(dse, s0f, s0e * dsf), (1.0f / 3.0f) * dse * dsf));
+}
+
+template <int SHAPE>
+__device__ __forceinline__ float esk_T(float s0e, float dse, float s0f, float dsf)
+{
+    if (SHAPE == 1)
+        return esk_T_cic(s0e, dse, s0f, dsf);
+    return fmaf(esk_A(s0e, dse), s0f, esk_B(s0e, dse) * dsf);
 }
 
 // ------------------------------------------------------------ fixed-point J tile
@@ -371,16 +389,6 @@ __device__ __forceinline__ float chunk_scale(int n, float bound, float* inv)
     return ldexpf(1.0f, hb - e);
 }
 
-// Esirkepov factor of two lines at once (packed FP32; per lane the same
-// operations as esk_T).
-__device__ __forceinline__ float2 esk_T2(float2 s0e, float2 dse, float2 s0f, float2 dsf)
-{
-    const float2 half = make_float2(0.5f, 0.5f), third = make_float2(1.0f / 3.0f, 1.0f / 3.0f);
-    return __ffma2_rn(s0e, s0f,
-                      __ffma2_rn(half, __ffma2_rn(dse, s0f, __fmul2_rn(s0e, dsf)),
-                                 __fmul2_rn(__fmul2_rn(third, dse), dsf)));
-}
-
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
 
 // One window line pair: the M - 1 terms P[i] T of two parallel lines (tile
@@ -397,103 +405,65 @@ __device__ __forceinline__ void add_line_pair(int* a0, int* a1, int st, const fl
     }
 }
 
+// One current component on a window of M nodes per axis (M - 1 half nodes
+// along the component's own axis d, whose DS are DSd): axis e carries the
+// factors A, B (times the component's coefficient cf), axis f its S0 and DS.
+// at: window origin of the component's tile; SD, SE, SF: word strides of the
+// three axes.  For PCS (144 atomics per move) the transverse factors and the fixed-point conversions go two lines at a time through the packed
+// FP32 pipe; for CIC and TSC the pairs' extra registers cost more than they
+// save.
+template <int SHAPE, int M, int SD, int SE, int SF>
+__device__ __forceinline__ void deposit_comp(int* at, float cf, const float* DSd, const float* S0e,
+                                             const float* DSe, const float* S0f, const float* DSf)
+{
+    constexpr bool PAIR = SHAPE == 3;
+    float P[M - 1], A[M], B[M];
+    P[0] = DSd[0];
+#pragma unroll
+    for (int i = 1; i < M - 1; ++i)
+        P[i] = P[i - 1] + DSd[i];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        A[j] = cf * esk_A(S0e[j], DSe[j]);
+        B[j] = cf * esk_B(S0e[j], DSe[j]);
+    }
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+        int j = 0;
+        if (PAIR) {
+#pragma unroll
+            for (; j + 1 < M; j += 2) {
+                const float2 T = __ffma2_rn(make_float2(A[j], A[j + 1]), dup2(S0f[k]),
+                                            __fmul2_rn(make_float2(B[j], B[j + 1]), dup2(DSf[k])));
+                add_line_pair<M>(at + k * SF + j * SE, at + k * SF + (j + 1) * SE, SD, P, T);
+            }
+        }
+#pragma unroll
+        for (; j < M; ++j) {
+            const float T = SHAPE == 1 ? cf * esk_T_cic(S0e[j], DSe[j], S0f[k], DSf[k])
+                                       : fmaf(A[j], S0f[k], B[j] * DSf[k]);
+            int* line = at + k * SF + j * SE;
+#pragma unroll
+            for (int i = 0; i < M - 1; ++i)
+                atomicAdd(line + i * SD, magic_int(P[i] * T));
+        }
+    }
+}
+
 // Deposit the three current components on a window of M nodes per axis
 // (M-1 half nodes along the current's own axis); node 0 of axis d sits at
-// tile index b[d].  cx..cz carry jcoef_d w times the chunk scale.  With
-// PAIR (PCS: 144 atomics per move) the transverse factors and the
-// fixed-point conversions go two lines at a time through the packed FP32
-// pipe; for CIC and TSC the pairs' extra registers cost more than they save.
-template <int M, int PX, int TY, int NJ, bool PAIR>
+// tile index b[d].  cx..cz carry jcoef_d w times the chunk scale.
+template <int SHAPE, int M, int PX, int TY, int NJ>
 __device__ __forceinline__ void deposit_window(int* sJi, const int b[3], const float* S0x,
                                                const float* S0y, const float* S0z, const float* DSx,
                                                const float* DSy, const float* DSz, float cx, float cy,
                                                float cz)
 {
     constexpr int PY = PX * TY;
-    {
-        float P[M - 1];
-        P[0] = DSx[0];
-#pragma unroll
-        for (int i = 1; i < M - 1; ++i)
-            P[i] = P[i - 1] + DSx[i];
-#pragma unroll
-        for (int k = 0; k < M; ++k)
-#pragma unroll
-            for (int j = 0; j < M; j += 2) {
-                int* row = sJi + (b[2] + k) * PY + (b[1] + j) * PX + b[0];
-                if (PAIR && j + 1 < M) {
-                    const float2 T = __fmul2_rn(dup2(cx), esk_T2(make_float2(S0y[j], S0y[j + 1]),
-                                                                make_float2(DSy[j], DSy[j + 1]),
-                                                                dup2(S0z[k]), dup2(DSz[k])));
-                    add_line_pair<M>(row, row + PX, 1, P, T);
-                } else {
-#pragma unroll
-                    for (int jj = j; jj < (PAIR ? j + 1 : min(j + 2, M)); ++jj) {
-                        const float T = cx * esk_T(S0y[jj], DSy[jj], S0z[k], DSz[k]);
-                        int* r = row + (jj - j) * PX;
-#pragma unroll
-                        for (int i = 0; i < M - 1; ++i)
-                            atomicAdd(r + i, magic_int(P[i] * T));
-                    }
-                }
-            }
-    }
-    {
-        float P[M - 1];
-        P[0] = DSy[0];
-#pragma unroll
-        for (int i = 1; i < M - 1; ++i)
-            P[i] = P[i - 1] + DSy[i];
-#pragma unroll
-        for (int k = 0; k < M; ++k)
-#pragma unroll
-            for (int i = 0; i < M; i += 2) {
-                int* col = sJi + NJ + (b[2] + k) * PY + b[1] * PX + (b[0] + i);
-                if (PAIR && i + 1 < M) {
-                    const float2 T = __fmul2_rn(dup2(cy), esk_T2(dup2(S0z[k]), dup2(DSz[k]),
-                                                                make_float2(S0x[i], S0x[i + 1]),
-                                                                make_float2(DSx[i], DSx[i + 1])));
-                    add_line_pair<M>(col, col + 1, PX, P, T);
-                } else {
-#pragma unroll
-                    for (int ii = i; ii < (PAIR ? i + 1 : min(i + 2, M)); ++ii) {
-                        const float T = cy * esk_T(S0z[k], DSz[k], S0x[ii], DSx[ii]);
-                        int* c = col + (ii - i);
-#pragma unroll
-                        for (int j = 0; j < M - 1; ++j)
-                            atomicAdd(c + j * PX, magic_int(P[j] * T));
-                    }
-                }
-            }
-    }
-    {
-        float P[M - 1];
-        P[0] = DSz[0];
-#pragma unroll
-        for (int i = 1; i < M - 1; ++i)
-            P[i] = P[i - 1] + DSz[i];
-#pragma unroll
-        for (int j = 0; j < M; ++j)
-#pragma unroll
-            for (int i = 0; i < M; i += 2) {
-                int* col = sJi + 2 * NJ + b[2] * PY + (b[1] + j) * PX + (b[0] + i);
-                if (PAIR && i + 1 < M) {
-                    const float2 T = __fmul2_rn(dup2(cz), esk_T2(make_float2(S0x[i], S0x[i + 1]),
-                                                                make_float2(DSx[i], DSx[i + 1]),
-                                                                dup2(S0y[j]), dup2(DSy[j])));
-                    add_line_pair<M>(col, col + 1, PY, P, T);
-                } else {
-#pragma unroll
-                    for (int ii = i; ii < (PAIR ? i + 1 : min(i + 2, M)); ++ii) {
-                        const float T = cz * esk_T(S0x[ii], DSx[ii], S0y[j], DSy[j]);
-                        int* c = col + (ii - i);
-#pragma unroll
-                        for (int k = 0; k < M - 1; ++k)
-                            atomicAdd(c + k * PY, magic_int(P[k] * T));
-                    }
-                }
-            }
-    }
+    int* at = sJi + b[2] * PY + b[1] * PX + b[0];
+    deposit_comp<SHAPE, M, 1, PX, PY>(at, cx, DSx, S0y, DSy, S0z, DSz);
+    deposit_comp<SHAPE, M, PX, PY, 1>(at + NJ, cy, DSy, S0z, DSz, S0x, DSx);
+    deposit_comp<SHAPE, M, PY, 1, PX>(at + 2 * NJ, cz, DSz, S0x, DSx, S0y, DSy);
 }
 
 // ------------------------------------------------------------ async copies
@@ -770,7 +740,7 @@ __device__ __forceinline__ void deposit_common(int* sJi, const Records<C>& r, in
         }
     }
     const float ws = r.w[e] * scale;
-    deposit_window<NW, T::PX, T::TY, T::N, SHAPE == 3>(sJi, b, S0[0], S0[1], S0[2], DS[0], DS[1], DS[2], jc[0] * ws,
+    deposit_window<SHAPE, NW, T::PX, T::TY, T::N>(sJi, b, S0[0], S0[1], S0[2], DS[0], DS[1], DS[2], jc[0] * ws,
                                            jc[1] * ws, jc[2] * ws);
 }
 
@@ -815,7 +785,7 @@ __device__ __forceinline__ void deposit_general_move(int* sJi, int l, const floa
         }
     }
     const float ws = w * scale;
-    deposit_window<M, T::PX, T::TY, T::N, SHAPE == 3>(sJi, b, S0[0], S0[1], S0[2], DS[0], DS[1], DS[2], jc[0] * ws,
+    deposit_window<SHAPE, M, T::PX, T::TY, T::N>(sJi, b, S0[0], S0[1], S0[2], DS[0], DS[1], DS[2], jc[0] * ws,
                                           jc[1] * ws, jc[2] * ws);
 }
 
@@ -893,7 +863,7 @@ __device__ __forceinline__ void deposit_general_warp(int* sJi, const Records<C>&
             P[i] = __shfl_sync(FULL, pv, (8 * c + i) & 31);
         if (L < LINES) {
             const float cf = (c == 0 ? jc[0] : (c == 1 ? jc[1] : jc[2])) * ws;
-            const float Tv = cf * esk_T(s0e, dse, s0f, dsf);
+            const float Tv = cf * esk_T<SHAPE>(s0e, dse, s0f, dsf);
             const int st_c = c == 0 ? 1 : (c == 1 ? PX : PY);
             const int st_e = ea == 0 ? 1 : (ea == 1 ? PX : PY);
             const int st_f = fa == 0 ? 1 : (fa == 1 ? PX : PY);
