@@ -13,13 +13,15 @@
 //     released ones;
 //   place: every waiting particle goes to slot abase[L] + rank of its list;
 //     the same launch lists the supercells that hold mobile particles for
-//     the next push;
-//   free_push: released frames go back on the free stack.
+//     the next push, and the released frames go back on the free stack;
+//   finish: the free stack's new height; every sort_every-th step, the TSC
+//     and PCS lists are sorted by nearest node / cell for the pushes to come.
 // Loading particles from the host uses the same path: a conversion kernel
 // fills the move buffer, then the maintenance places them.
 #include "pic_internal.cuh"
 
 #include <cmath>
+#include <cstddef>
 
 namespace pic {
 
@@ -218,6 +220,9 @@ __global__ void __launch_bounds__(256) k_place(const StepDev d)
     if (tot.y > *d.free_top)
         return;
     list_items(d);
+    // the released frames take the places of those that k_scan_apply popped
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < tot.z; i += gridDim.x * blockDim.x)
+        d.free_stack[*d.free_top - tot.y + i] = d.released[i];
     const int n = min(*d.mv_count, d.mv_cap);
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n; m += gridDim.x * blockDim.x) {
         const int L = d.mv_dest[m];
@@ -237,20 +242,196 @@ __global__ void __launch_bounds__(256) k_place(const StepDev d)
     }
 }
 
-__global__ void __launch_bounds__(1024) k_free_push(const StepDev d)
+// ------------------------------------------------------------ list sort
+//
+// Sorts the frame lists of the mobile TSC and PCS species by nearest node (TSC)
+// or cell (PCS) in place, whole lists where they fit a run of kSortRun particles:
+// the run comes into shared memory by 16-byte asynchronous copies, a counting
+// sort gives every sorted position its source, and the attributes go back as
+// contiguous words.  Bound by HBM: 32 B per particle read and 32 B written.
+// Against sorting each chunk of 256 by itself inside the push, a warp of the
+// push reads fewer different field words (a bank model of the 8x4x4 TSC tile
+// at 8 particles per cell: 1.34 against 1.90 wavefronts per load), and the push
+// needs neither the sort's shared memory nor its four barriers per chunk.  256^3
+// cells, 8 TSC particles each: push 9.73 -> 8.72 ms per step, maintenance 0.19
+// -> 0.57 ms (a sort every fourth step takes 1.5 ms, 5.6 TB/s); 128^3 at 16 each
+// 2.28 + 0.11 -> 1.99 + 0.20 ms; PCS 96^3 1.26 + 0.07 -> 1.19 + 0.09 ms.
+// (CIC lists: see the sort in push_list, k_push.cu.)
+constexpr int kSortThreads = 256;
+constexpr int kSortRun = 1536;
+constexpr int kSortKeys = 1024;  // >= 729, the nodes of the largest supercell
+
+struct SortSmem {
+    int off[kSortKeys];             // histogram, then first sorted position of each key
+    unsigned short src[kSortRun];   // sorted position -> run position
+    int warp_sum[kSortThreads / 32];
+    unsigned st[8][kSortRun];       // cell, offsets, momenta, weight in run order
+    unsigned pid[kSortRun];         // ids; allocated only when they are tracked
+};
+
+static size_t sort_smem_bytes(bool ids) { return ids ? sizeof(SortSmem) : offsetof(SortSmem, pid); }
+
+__device__ __forceinline__ void sort_copy16(void* smem, const void* gmem)
 {
-    const int4 tot = *d.totals;
-    const int top = *d.free_top;
-    if (tot.y > top)
-        return;
-    const int base = top - tot.y;
-    for (int i = threadIdx.x; i < tot.z; i += blockDim.x)
-        d.free_stack[base + i] = d.released[i];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        *d.free_top = base + tot.z;
-        *d.mv_count = 0;
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+
+// base: a multiple of 4 (16-byte pieces of whole frames, which are allocated
+// even past the list's count)
+__device__ __forceinline__ void sort_run(const StepDev& d, SortSmem& sm, const int* ft, int base, int cn, int shape)
+{
+    const int tid = threadIdx.x;
+    const int LX = d.LX, LY = d.LY, LZ = d.LZ;  // powers of two
+    const int bx = __ffs(LX) - 1, by = __ffs(LY) - 1;
+    auto gidx = [&](int slot) -> int64_t { return (int64_t)ft[slot >> d.log2S] * d.S + (slot & (d.S - 1)); };
+    unsigned* const attr[8] = {reinterpret_cast<unsigned*>(d.cell), reinterpret_cast<unsigned*>(d.ox),
+                               reinterpret_cast<unsigned*>(d.oy),   reinterpret_cast<unsigned*>(d.oz),
+                               reinterpret_cast<unsigned*>(d.ux),   reinterpret_cast<unsigned*>(d.uy),
+                               reinterpret_cast<unsigned*>(d.uz),   reinterpret_cast<unsigned*>(d.w)};
+    for (int k = tid; k < (cn + 3) >> 2; k += kSortThreads) {
+        const int64_t idx = gidx(base + 4 * k);
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+            sort_copy16(sm.st[a] + 4 * k, attr[a] + idx);
+        if (d.pid)
+            sort_copy16(sm.pid + 4 * k, d.pid + idx);
     }
+    const int K = shape == 2 ? (LX + 1) * (LY + 1) * (LZ + 1) : d.S;
+    for (int k = tid; k < K; k += kSortThreads)
+        sm.off[k] = 0;
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    constexpr int Q = kSortRun / kSortThreads;
+    int kr[Q];  // of this thread's particles: key << 16 | rank within the key
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int j = q * kSortThreads + tid;
+        if (j >= cn)
+            break;
+        const int cell = (int)sm.st[0][j];
+        int key = cell;
+        if (shape == 2) {
+            const int lx = (cell & (LX - 1)) + (__uint_as_float(sm.st[1][j]) >= 0.5f);
+            const int ly = ((cell >> bx) & (LY - 1)) + (__uint_as_float(sm.st[2][j]) >= 0.5f);
+            const int lz = (cell >> (bx + by)) + (__uint_as_float(sm.st[3][j]) >= 0.5f);
+            key = lx + (LX + 1) * (ly + (LY + 1) * lz);
+        }
+        kr[q] = (key << 16) | atomicAdd(&sm.off[key], 1);
+    }
+    __syncthreads();
+    // exclusive prefix of the histogram: every thread takes kSortKeys /
+    // kSortThreads keys in a row
+    {
+        constexpr int P = kSortKeys / kSortThreads;
+        const int lane = tid & 31, wid = tid >> 5;
+        int v[P], local = 0;
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            const int k = P * tid + i;
+            v[i] = k < K ? sm.off[k] : 0;
+            local += v[i];
+        }
+        int incl = local;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o)
+                incl += y;
+        }
+        if (lane == 31)
+            sm.warp_sum[wid] = incl;
+        __syncthreads();
+        int run = incl - local;
+        for (int w = 0; w < wid; ++w)
+            run += sm.warp_sum[w];
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            const int k = P * tid + i;
+            if (k < K)
+                sm.off[k] = run;
+            run += v[i];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int j = q * kSortThreads + tid;
+        if (j < cn)
+            sm.src[sm.off[kr[q] >> 16] + (kr[q] & 0xffff)] = (unsigned short)j;
+    }
+    __syncthreads();
+    for (int j = tid; j < cn; j += kSortThreads) {
+        const int64_t idx = gidx(base + j);
+        const int from = sm.src[j];
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+            attr[a][idx] = sm.st[a][from];
+        if (d.pid)
+            d.pid[idx] = (int)sm.pid[from];
+    }
+    __syncthreads();  // the next run fills the stage and clears the histogram
+}
+
+__device__ __forceinline__ void sort_lists(const StepDev& d, SortSmem& sm, const int* foff, const int* ftab, int first,
+                                           int stride)
+{
+    const int nitems = *d.nitems;
+    for (int t = first; t < nitems * d.nspecies; t += stride) {
+        const int s = t / nitems;
+        const int L = s * d.nsc + d.items[t - s * nitems];
+        const int n = d.count[L];
+        const int shape = d.sp[s].shape;
+        if (!d.sp[s].mobile || shape == 1 || n <= 1)
+            continue;
+        const int runs = (n + kSortRun - 1) / kSortRun;
+        const int per = ((n + runs - 1) / runs + 31) & ~31;
+        for (int base = 0; base < n; base += per)
+            sort_run(d, sm, ftab + foff[L], base, min(per, n - base), shape);
+    }
+}
+
+// The lists in the current frame table, before the first push after a load.
+__global__ void __launch_bounds__(kSortThreads) k_sort(const StepDev d)
+{
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    sort_lists(d, *reinterpret_cast<SortSmem*>(sort_smem), d.foff, d.ftab, (int)blockIdx.x, (int)gridDim.x);
+}
+
+// Last kernel of the maintenance: block 0 settles the free stack and the move
+// buffer; on every sort_every-th step the others sort the lists (the frame
+// table written in this step is the current one from here on).
+__global__ void __launch_bounds__(kSortThreads) k_finish(const StepDev d)
+{
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) {
+            const int4 tot = *d.totals;
+            const int top = *d.free_top;
+            if (tot.y <= top) {
+                *d.free_top = top - tot.y + tot.z;
+                *d.mv_count = 0;
+            }
+        }
+        return;
+    }
+    if (*d.step_ctr % d.sort_every == 0)
+        sort_lists(d, *reinterpret_cast<SortSmem*>(sort_smem), d.foff_next, d.ftab_next, (int)blockIdx.x - 1,
+                   (int)gridDim.x - 1);
+}
+
+cudaError_t configure_sort()
+{
+    cudaError_t e = cudaFuncSetAttribute(k_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem));
+    return e;
+}
+
+cudaError_t launch_sort(const StepDev& d, int blocks, cudaStream_t st)
+{
+    k_sort<<<blocks, kSortThreads, sort_smem_bytes(d.pid != nullptr), st>>>(d);
+    return cudaGetLastError();
 }
 
 // Moving window, part 1: empty the lists of the bottom `rows` supercell
@@ -313,12 +494,12 @@ cudaError_t launch_frame_plan(const StepDev& d, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_frame_apply(const StepDev& d, int place_blocks, cudaStream_t st)
+cudaError_t launch_frame_apply(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st)
 {
     const int nblk = frame_scan_blocks(d.nlists);
     k_scan_apply<<<nblk, kScanThreads, 0, st>>>(d);
     k_place<<<place_blocks, 256, 0, st>>>(d);
-    k_free_push<<<1, 1024, 0, st>>>(d);
+    k_finish<<<1 + sort_blocks, kSortThreads, sort_blocks > 0 ? sort_smem_bytes(d.pid != nullptr) : 0, st>>>(d);
     return cudaGetLastError();
 }
 

@@ -31,16 +31,17 @@
 //                     * [S0y S0z + DSy S0z / 2 + S0y DSz / 2 + DSy DSz / 3](j, k)
 // i.e. an outer product of a prefix sum along x and a transverse factor.
 //
-// Particles go through a chunk of at most 256 at a time in the order of a
-// counting sort by nearest node (cell for CIC and PCS), so the lanes of a
-// warp read neighbouring field words (shared-memory broadcasts).  Every
-// sort_every-th step (a sort pass) stages each chunk in shared memory, sorts
-// it and writes it back to the list in sorted order; the steps between push
-// the lists in stored order from the chunk stage, which an asynchronous copy
-// fills while the previous chunk deposits.  The push writes a deposit record
+// Particles go through a chunk of at most 256 at a time in list order.  Every
+// sort_every-th step the frame maintenance sorts the TSC and PCS lists by
+// nearest node / cell, so the lanes of a warp read neighbouring field words
+// (shared-memory broadcasts) and a chunk covers a few rows of nodes.  CIC lists
+// are sorted here, chunk by chunk by cell, in the push of that step (a sort
+// pass; see push_list).  The chunk stage is filled by an asynchronous copy while
+// the previous chunk deposits (in a CIC sort pass by plain loads).
+// The push writes a deposit record
 // per particle; the deposit then runs in a lane order whose neighbours are
-// kDepStride sorted positions apart, so one warp's atomics land on different
-// nodes.  The current of a chunk accumulates in fixed point (see
+// several list positions apart (dep_log_stride), so one warp's atomics land on
+// different nodes.  The current of a chunk accumulates in fixed point (see
 // chunk_scale).  Two deposit paths, both exact forms of that formula:
 //   common: on every axis the move stays on one spline piece -- the old and
 //     the new position round to the same node (TSC) / stay in the same cell
@@ -71,10 +72,14 @@ constexpr int kGenDefer = 64;
 // to the move buffer at the start of its next work item (more go straight
 // to the move buffer).
 constexpr int kLeaverBuf = 48;
-// Lane stride of the deposit over the node-sorted chunk: 4 spreads one
-// warp's 54 atomics per particle over the banks better than 1 (neighbours
-// share a node) or C / 32 (random over the tile).
-constexpr int kDepStride = 4;
+// Log2 of the lane stride of the deposit over a chunk of a list of n
+// particles in a supercell of S cells: neighbouring lanes take list positions
+// that far apart, so that one warp's atomics land on different nodes.  The
+// list is sorted by node, with n / S particles on a node on average; in a bank
+// model of the 8x4x4 tile a TSC atomic of 32 lanes takes 3.1 / 3.3 / 4.8
+// wavefronts at stride 4 and 3.3 / 2.9 / 3.1 at stride 8 for 2 / 8 / 16
+// particles per cell.
+__device__ __forceinline__ int dep_log_stride(int n, int S) { return n >= 4 * S ? 3 : 2; }
 
 // G = guard cells below the supercell (the fields' global guards match):
 // 1 for CIC/TSC, 2 when a PCS species is present (its support reaches two
@@ -338,11 +343,9 @@ __device__ __forceinline__ float2 gather_pair(const float* __restrict__ F1, int 
 // Esirkepov's transverse factor S0e S0f + (DSe S0f + S0e DSf)/2 + DSe DSf / 3
 // as A S0f + B DSf with A = S0e + DSe / 2, B = S0e / 2 + DSe / 3: A and B
 // belong to one node of axis e, so that a line of the window takes two
-// operations instead of seven (27 lines per TSC move; the TSC push of 256^3
-// cells at 8 particles each went from 9.97 to 9.73 ms).  CIC moves (12 lines
-// in the common window) keep the form of esk_T_cic and its rounding: the
-// energy-conserving CIC gather jumps at half a cell, where another rounding of
-// the current now and then gives a particle another kick.
+// operations instead of seven (27 lines per TSC move).  CIC moves (12 lines
+// in the common window) keep the form of esk_T_cic and its rounding: see the
+// sort in push_list.
 __device__ __forceinline__ float esk_A(float s0, float ds) { return fmaf(0.5f, ds, s0); }
 __device__ __forceinline__ float esk_B(float s0, float ds) { return fmaf(0.5f, s0, (1.0f / 3.0f) * ds); }
 
@@ -531,23 +534,23 @@ __device__ __forceinline__ void warp_exclusive_scan_counts(const int* cnt, int* 
 // ------------------------------------------------------------ shared state
 
 // Particles of one chunk of a frame list, staged in shared memory in list
-// order, plus their counting-sort permutation by nearest node.
+// order, and, for the sort passes of CIC lists, their counting-sort
+// permutation by cell.
 template <int C, bool PCS>
 struct Stage {
     int cell[C];
     float o[3][C];
     float u[3][C];
     float w[C];
-    int pid[C];   // particle ids (only when tracked)
+    int pid[C];   // particle ids (sort passes, only when tracked)
     int kr[C];    // key << 16 | rank within key
     int perm[C];  // sorted position -> chunk position
     int brk[PCS ? C : 1];  // PCS, by push position: bank << 16 | rank within the bank
 };
 
-// Deposit inputs of the chunk's moves, by sorted position s stored at slot
-// rslot(s) = s + s / 32: the deposit reads them with a stride of
-// kDepStride between lanes, and the skew puts the 32 lanes on 32 different
-// banks.
+// Deposit inputs of the chunk's moves, by chunk position s stored at slot
+// rslot(s) = s + s / 32: the deposit reads them with a stride of 4 or 8
+// between lanes, and the skew puts the 32 lanes on 32 different banks.
 __host__ __device__ constexpr int rslot(int s) { return s + (s >> 5); }
 
 // PCS (144 atomics per common-window move): the chunk's moves are
@@ -574,19 +577,8 @@ struct Records {
     float o[3][R];   // old in-cell offsets
     float D[3][R];   // displacement in cells
     float w[R];      // weight
-    int gen[C];      // sorted positions of the moves that need the general window
+    int gen[C];      // chunk positions of the moves that need the general window
 };
-
-template <class T, int SHAPE>
-struct Keys {
-    static constexpr int K = SHAPE == 2 ? (T::LX + 1) * (T::LY + 1) * (T::LZ + 1) : T::S;
-};
-
-template <class T>
-constexpr int max_keys()
-{
-    return (T::LX + 1) * (T::LY + 1) * (T::LZ + 1);
-}
 
 // General-window moves set aside for one lane-parallel deposit after the
 // last chunk of a frame list (the few of each chunk would otherwise keep one
@@ -616,8 +608,8 @@ struct SharedState {
     Records<C> rec;
     GenDefer gd;
     LeaverBuf lv;
-    int hist[max_keys<T>()];
-    int off[max_keys<T>()];
+    int hist[T::S];  // sort passes: particles per cell, and each cell's first sorted position
+    int off[T::S];
     unsigned long long mb_tile;    // completion of the E/B tile's tensor loads
     unsigned alive[NQ * NT / 32];  // per warp and pass: ballot of the pushed particles that stay
     int item, nlv, lv_base;
@@ -660,8 +652,7 @@ __device__ __forceinline__ int dealt_slot(const int* brk, int sidx, int cn, int 
     return deal_slot<C>(__shfl_sync(0xffffffffu, boff, br >> 16) + (br & 0xffff));
 }
 
-// Stored-order passes: start copying the particles of list slots
-// [base, base + cn) into the chunk stage (cell, offsets, momenta, weight;
+// Start copying the particles of list slots [base, base + cn) into the chunk stage (cell, offsets, momenta, weight;
 // 16-byte pieces of whole frames, which are allocated even past the list's
 // count).  The caller waits with cp_async_wait_all and a block barrier.
 template <class T, int NT>
@@ -789,7 +780,7 @@ __device__ __forceinline__ void deposit_general_move(int* sJi, int l, const floa
                                           jc[1] * ws, jc[2] * ws);
 }
 
-// The general-window move at sorted position s of the chunk's records.
+// The general-window move at position s of the chunk's records.
 template <class T, int SHAPE, int C>
 __device__ __forceinline__ void deposit_general(int* sJi, const Records<C>& r, int s, const float jc[3],
                                                 float scale)
@@ -1159,9 +1150,9 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
                                           const float* sF, int* sJi, float* sJf,
                                           SharedState<T, NT>& sh, bool sort_pass, unsigned& my_status)
 {
-    constexpr int LX = T::LX, LY = T::LY, S = T::S, N = T::N;
+    constexpr int S = T::S, N = T::N;
+    constexpr bool SORTS = SHAPE == 1;  // sorted in the push, chunk by chunk
     constexpr int C = SharedState<T, NT>::C;
-    constexpr int K = Keys<T, SHAPE>::K;
     constexpr bool DEAL = SHAPE == 3;  // bank-dealt deposit slots (see deal_slot)
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int L = s * d.nsc + g;
@@ -1169,6 +1160,9 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
     const int* ft = d.ftab + d.foff[L];
     auto gidx = [&](int slot) -> int64_t { return (int64_t)ft[slot >> d.log2S] * S + (slot & (S - 1)); };
     constexpr int NQ = SharedState<T, NT>::NQ, NWARP = NT / 32;
+    constexpr int kLogC = C == 256 ? 8 : 7;
+    static_assert(C == 1 << kLogC, "a chunk is 128 or 256 particles");
+    const int ls = SORTS ? 2 : dep_log_stride(n, S);
     float prev_inv = 0.0f;
     int ndef = 0;  // general-window moves set aside in sh.gd
     int surv = 0;  // particles of the list that stay, written back so far
@@ -1182,53 +1176,47 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
         if (base > 0)
             fold_tile<N, NT>(sJi, sJf, prev_inv);  // previous chunk; the push below does not touch J
         int boff = 0;
-        if (sort_pass) {
-            // stage the chunk (coalesced), key = nearest node (TSC) / cell (CIC),
-            // then a counting sort; the pushed particles go back to the list
-            // in sorted order, so the list stays sorted by node between passes
-            for (int k = tid; k < K; k += NT)
+        const bool sort = SORTS && sort_pass;
+        if (sort) {
+            // CIC: stage the chunk (coalesced), key = cell, then a counting
+            // sort; the pushed particles go back to the list in sorted order.
+            // Against a sort of the whole lists by the frame maintenance (as
+            // for TSC and PCS) this costs no extra pass over the particles, and
+            // CIC gains little from whole-list order (128^3, 8 per cell, push +
+            // maintenance: 0.842 ms this way, 0.864 ms with the lists sorted
+            // there).  It also keeps the particles of every chunk together,
+            // and with them the fixed-point scale of its current: the
+            // energy-conserving CIC gather jumps at half a cell, where another
+            // rounding now and then gives a particle another kick.
+            for (int k = tid; k < S; k += NT)
                 sh.hist[k] = 0;
             __syncthreads();
             for (int j = tid; j < cn; j += NT) {
                 const int64_t idx = gidx(base + j);
                 const int cell = d.cell[idx];
-                const float ox = d.ox[idx], oy = d.oy[idx], oz = d.oz[idx];
                 sh.st.cell[j] = cell;
-                sh.st.o[0][j] = ox;
-                sh.st.o[1][j] = oy;
-                sh.st.o[2][j] = oz;
+                sh.st.o[0][j] = d.ox[idx];
+                sh.st.o[1][j] = d.oy[idx];
+                sh.st.o[2][j] = d.oz[idx];
                 sh.st.u[0][j] = d.ux[idx];
                 sh.st.u[1][j] = d.uy[idx];
                 sh.st.u[2][j] = d.uz[idx];
                 sh.st.w[j] = d.w[idx];
                 if (d.pid)
                     sh.st.pid[j] = d.pid[idx];
-                int key;
-                if (SHAPE == 2) {
-                    const int lx = cell % LX + (ox >= 0.5f), ly = (cell / LX) % LY + (oy >= 0.5f),
-                              lz = cell / (LX * LY) + (oz >= 0.5f);
-                    key = lx + (LX + 1) * (ly + (LY + 1) * lz);
-                } else {
-                    key = cell;
-                }
-                sh.st.kr[j] = (key << 16) | atomicAdd(&sh.hist[key], 1);
+                sh.st.kr[j] = (cell << 16) | atomicAdd(&sh.hist[cell], 1);
             }
             __syncthreads();
             if (wid == 0)
-                warp_exclusive_scan_counts(sh.hist, sh.off, K);
+                warp_exclusive_scan_counts(sh.hist, sh.off, S);
             __syncthreads();
             for (int j = tid; j < cn; j += NT) {
                 const int kr = sh.st.kr[j];
-                const int ps = sh.off[kr >> 16] + (kr & 0xffff);
-                sh.st.perm[ps] = j;
-                if (DEAL) {
-                    const int bk = dep_bank<T>(sh.st.cell[j]);
-                    sh.st.brk[ps] = (bk << 16) | atomicAdd(&sh.bh[bk], 1);
-                }
+                sh.st.perm[sh.off[kr >> 16] + (kr & 0xffff)] = j;
             }
             __syncthreads();
-            boff = DEAL ? bank_offsets(sh.bh, lane) : 0;
-        } else if (DEAL) {
+        }
+        if (DEAL) {
             for (int j = tid; j < cn; j += NT) {
                 const int bk = dep_bank<T>(sh.st.cell[j]);
                 sh.st.brk[j] = (bk << 16) | atomicAdd(&sh.bh[bk], 1);
@@ -1236,9 +1224,8 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
             __syncthreads();
             boff = bank_offsets(sh.bh, lane);
         }
-        // push: sort passes in sorted order (neighbouring lanes read
-        // neighbouring field words), the passes between in stored order from
-        // the stage an async copy filled while the previous chunk deposited.
+        // push, from the stage that an async copy filled while the previous
+        // chunk deposited.
         // Every read of the chunk's list slots happens before the barrier
         // below, every write after it.
         Part qs[NQ];
@@ -1250,7 +1237,7 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
             float bnd = 0.0f;
             qs[r].cell = -1;
             if (sidx < cn) {
-                const int j = sort_pass ? sh.st.perm[sidx] : sidx;
+                const int j = sort ? sh.st.perm[sidx] : sidx;
                 Part& q = qs[r];
                 q.cell = sh.st.cell[j];
                 q.o[0] = sh.st.o[0][j];
@@ -1260,7 +1247,7 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
                 q.u[1] = sh.st.u[1][j];
                 q.u[2] = sh.st.u[2][j];
                 q.w = sh.st.w[j];
-                pids[r] = !d.pid ? 0 : (sort_pass ? sh.st.pid[j] : d.pid[gidx(base + sidx)]);
+                pids[r] = !d.pid ? 0 : (sort ? sh.st.pid[j] : d.pid[gidx(base + sidx)]);
                 bnd = push_one<T, SHAPE, NT>(d, sp, s, bx, scx, scy, scz, sF, sh, q, pids[r], slot, cb,
                                              my_status);
             }
@@ -1273,7 +1260,7 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
         }
         __syncthreads();
         // the particles that stay go back to the list compacted, in chunk
-        // order (the leavers' slots close up; sorted lists stay sorted)
+        // order (the leavers' slots close up; sorted lists stay nearly sorted)
         {
             int run = 0, pre[NQ];
 #pragma unroll
@@ -1289,7 +1276,7 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
                     continue;
                 const int src = base + r * NT + tid;
                 const int dst = surv + pre[r] + __popc(sh.alive[r * NWARP + wid] & ((1u << lane) - 1u));
-                const bool moved = sort_pass || dst != src;
+                const bool moved = sort || dst != src;
                 const int64_t idx = gidx(dst);
                 store_part(d, idx, qs[r], moved);
                 if (d.pid && moved)
@@ -1303,16 +1290,16 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
         }
         if (DEAL && T::G == 2 && tid < 32)
             sh.bh[tid] = 0;  // every warp read it before the barrier above; next written after the chunk
-        if (!sort_pass && base + C < n)  // the stage is free: the next chunk flies during the deposit
+        if (!sort && base + C < n)  // the stage is free: the next chunk flies during the deposit
             stage_chunk_async<T, NT>(d, sh, L, base + C, min(C, n - base - C));
-        // deposit: neighbouring lanes take chunk positions kDepStride apart
-        // (sorted by node, so one warp's atomics land on different nodes and
-        // mostly different banks); then the general-window moves
+        // deposit: neighbouring lanes take chunk positions 1 << ls apart (the
+        // list is sorted by node, so one warp's atomics land on different nodes
+        // and mostly different banks); then the general-window moves
         float inv;
         const float scale = chunk_scale(cn, __uint_as_float(sh.bound_bits[cb]), &inv);
         for (int r = 0; r < C / NT; ++r) {
             const int q = r * NT + tid;
-            const int e = DEAL ? q : kDepStride * (q % (C / kDepStride)) + q / (C / kDepStride);
+            const int e = DEAL ? q : ((q << ls) & (C - 1)) + (q >> (kLogC - ls));
             if ((DEAL ? deal_pos<C>(q) : e) < cn && !(sh.rec.l[rslot(e)] >> 24))
                 deposit_common<T, SHAPE, C>(sJi, sh.rec, e, sp.jcoef, scale);
         }
@@ -1346,8 +1333,7 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
                 deposit_general_warp<T, SHAPE, C>(sJi, sh.rec, sh.rec.gen[nfull + t], sp.jcoef, scale);
         }
         prev_inv = inv;
-        if (!sort_pass)
-            cp_async_wait_all();
+        cp_async_wait_all();
         __syncthreads();
     }
     if (n > 0)
@@ -1387,10 +1373,9 @@ __global__ void __launch_bounds__(NT, (T::G == 1 ? 1024 : 512) / NT) k_push_depo
 
     const int tid = threadIdx.x;
     unsigned my_status = 0;
-    // every sort_every-th step reorders the lists (the counter only changes
-    // between launches, so all CTAs agree)
-    const bool sort_pass = d.sort_every <= 1 || (*d.step_ctr % d.sort_every) == 0;
-
+    // every sort_every-th step reorders the lists; CIC lists here (the counter
+    // only changes between launches, so all CTAs agree)
+    const bool sort_pass = *d.step_ctr % d.sort_every == 0;
     // work items: tid 0 asks for the next one while the block works on the
     // current one, and publishes it at the end of the item
     if (tid == 0) {
@@ -1425,18 +1410,16 @@ __global__ void __launch_bounds__(NT, (T::G == 1 ? 1024 : 512) / NT) k_push_depo
         if (tid == 0)
             sh.nlv = 0;  // every thread read it in flush_leavers (before its barrier, if it had one)
 
-        // ---- 1. the E/B tile by two tensor loads (TMA); on a stored-order
-        // pass the first chunk of the first mobile list is copied meanwhile;
-        // the next work item's tile is prefetched into L2; the J tiles are
-        // zeroed
+        // ---- 1. the E/B tile by two tensor loads (TMA); the first chunk of
+        // the first mobile list is copied meanwhile; the next work item's tile
+        // is prefetched into L2; the J tiles are zeroed
         int pre_s = -1;
-        if (!sort_pass) {
-            for (int s = 0; s < d.nspecies && pre_s < 0; ++s) {
-                const int n = d.count[s * d.nsc + g];
-                if (d.sp[s].mobile && n > 0) {
-                    pre_s = s;
+        for (int s = 0; s < d.nspecies && pre_s < 0; ++s) {
+            const int n = d.count[s * d.nsc + g];
+            if (d.sp[s].mobile && n > 0) {
+                pre_s = s;
+                if (!(sort_pass && d.sp[s].shape == 1))
                     stage_chunk_async<T, NT>(d, sh, s * d.nsc + g, 0, min(SharedState<T, NT>::C, n));
-                }
             }
         }
         if (tid == 0) {
@@ -1482,11 +1465,9 @@ __global__ void __launch_bounds__(NT, (T::G == 1 ? 1024 : 512) / NT) k_push_depo
                 sh.bound_bits[0] = 0u;
                 sh.gd_bound_bits = 0u;
             }
-            if (!sort_pass) {
-                if (s != pre_s)
-                    stage_chunk_async<T, NT>(d, sh, L, 0, min(SharedState<T, NT>::C, n));
-                cp_async_wait_all();
-            }
+            if (s != pre_s && !(sort_pass && sp.shape == 1))
+                stage_chunk_async<T, NT>(d, sh, L, 0, min(SharedState<T, NT>::C, n));
+            cp_async_wait_all();
             __syncthreads();
             int stay;
             if (sp.shape == 2)

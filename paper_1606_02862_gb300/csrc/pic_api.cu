@@ -98,7 +98,7 @@ struct pic_ctx {
           *mv_uz = nullptr, *mv_w = nullptr;
     int4 *blk_sums = nullptr, *blk_offs = nullptr, *totals = nullptr;
     int* work_counter = nullptr;
-    int* step_ctr = nullptr;           // device step count, read by the push for its sort passes
+    int* step_ctr = nullptr;           // device step count since the last load (when the lists are sorted)
     long long* step_no = nullptr;      // device: steps taken since creation (antenna time)
     int64_t steps_done = 0;            // host: steps enqueued since creation
     int64_t host_direct = 0;           // load / read calls that converted page-locked host arrays in place
@@ -588,7 +588,7 @@ pic_status enqueue_stage(pic_ctx* c, int stage, int parity, int fsrc = -1)
         return PIC_OK;
     case PIC_STAGE_FRAMES:
         CK(launch_frame_plan(d, c->stream));
-        CK(launch_frame_apply(d, 4 * c->nsm, c->stream));
+        CK(launch_frame_apply(d, 4 * c->nsm, 4 * c->nsm, c->stream));
         return PIC_OK;
     default:
         CK(launch_yee_mixed_part(yee_plan(c), stage - PIC_STAGE_B_FIRST, c->stream));
@@ -647,6 +647,9 @@ pic_status prepare_mixed(pic_ctx* c)
     int per_sm = 0;
     CK(configure_push(c->LX, c->LY, c->LZ, c->threads, c->guard, &per_sm));
     c->push_grid = std::max(1, per_sm) * c->nsm;
+    // freshly loaded particles sit unsorted at the ends of their lists
+    CK(configure_sort());
+    CK(launch_sort(make_step(c, c->parity), 4 * c->nsm, c->stream));
     CKS(prepare_fused(c));
     c->prepared = true;
     return PIC_OK;
@@ -1428,7 +1431,7 @@ pic_status pic_shift_window(pic_ctx* c, int32_t box, int32_t cells)
     CK(launch_clear_rows(d, b, rows, c->stream));
     CK(cudaMemsetAsync(c->mv_count, 0, sizeof(int), c->stream));
     CK(launch_frame_plan(d, c->stream));
-    CK(launch_frame_apply(d, 4 * c->nsm, c->stream));
+    CK(launch_frame_apply(d, 4 * c->nsm, 0, c->stream));
     CKS(status_check(c));
     c->parity ^= 1;
     if (!c->rot_scratch)
@@ -1577,8 +1580,8 @@ pic_status insert_mixed(pic_ctx* c, int box, int species, int64_t m, const doubl
                 return fail(c, PIC_ERR_ARG, "non-finite particle data");
             }
             // count the frames this insertion needs, grow the pool, then place;
-            // the next step is a sort pass (the arrivals sit unsorted at the
-            // list ends)
+            // the lists are sorted before the next step (the arrivals sit
+            // unsorted at the list ends)
             d.step_ctr = nullptr;
             CK(cudaMemsetAsync(c->step_ctr, 0, sizeof(int), c->stream));
             CK(launch_frame_plan(d, c->stream));
@@ -1589,7 +1592,7 @@ pic_status insert_mixed(pic_ctx* c, int box, int species, int64_t m, const doubl
             if (tot.y > top)
                 CKS(ensure_pool(c, (c->pool_cap - top) + tot.y));
             d = make_step(c, c->parity);
-            CK(launch_frame_apply(d, 4 * c->nsm, c->stream));
+            CK(launch_frame_apply(d, 4 * c->nsm, 0, c->stream));
             CKS(status_check(c));
             c->parity ^= 1;
         }
@@ -1912,7 +1915,7 @@ pic_status build_like(pic_ctx* c, const TuneCfg& cfg, const TuneSnapshot& snap, 
 }
 
 // Push + frame maintenance milliseconds per step of configuration cfg on
-// the snapshot: after one warm-up step (the sort pass that follows a load),
+// the snapshot: after one warm-up step,
 // two whole sort periods timed with the step's stage events, so that sort
 // and stored-order passes weigh as they do in a run.
 double time_config(pic_ctx* c, const TuneCfg& cfg, const TuneSnapshot& snap)

@@ -39,7 +39,7 @@
 namespace pic {
 
 constexpr int kMaxSpecies = 8;
-constexpr int kDefaultSortEvery = 4;  // steps between sort passes of the push (mixed form)
+constexpr int kDefaultSortEvery = 4;  // steps between sorts of the frame lists (mixed form)
 constexpr int kYeeCellsZ = 4;         // cells per thread along z in the Yee kernels
 
 // Device status word bits (OR-ed by kernels, read by the host after a step).
@@ -148,7 +148,7 @@ struct StepDev {
     int* work_counter;        // persistent-kernel work counter
     int* step_ctr;            // device step count (advanced by the frame plan)
     long long* step_no;       // steps taken since creation (advanced with step_ctr, never reset)
-    int sort_every;           // the push sorts the frame lists every this many steps
+    int sort_every;           // the frame lists are sorted every this many steps
     unsigned* status;         // device status word
     unsigned* wmax_bits;      // [kMaxSpecies] float bits of the largest |weight| loaded
 };
@@ -231,7 +231,13 @@ int push_supported(int LX, int LY, int LZ, int threads, int guard);
 size_t push_smem_bytes(int LX, int LY, int LZ, int threads, int guard);
 int frame_scan_blocks(int nlists);
 cudaError_t launch_frame_plan(const StepDev& d, cudaStream_t st);
-cudaError_t launch_frame_apply(const StepDev& d, int place_blocks, cudaStream_t st);
+// sort_blocks > 0: blocks that sort the lists when the step count says so
+// (d.step_ctr; configure_sort called before)
+cudaError_t launch_frame_apply(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st);
+// the sort's shared-memory limit (call once, outside stream capture), and a
+// sort of every list now
+cudaError_t configure_sort();
+cudaError_t launch_sort(const StepDev& d, int blocks, cudaStream_t st);
 // ids: per-particle ids (or null: id_base + i)
 cudaError_t launch_insert_convert(const StepDev& d, int box, int species, int64_t n,
                                   const double* x, const double* u, const double* w,

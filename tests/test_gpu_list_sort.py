@@ -1,0 +1,42 @@
+"""The sort of the frame lists (TSC, PCS: whole lists in runs of at most 1536
+particles, by the frame maintenance; CIC: chunk by chunk in the push): one
+supercell holds n particles, n at the edges of a chunk (256), of a run and of
+two and three runs, the others a few.  The particles are the same after sorts
+on every step (ids, weights), and one step from the read-back state matches
+the FP64 oracle at the per-step tolerance of the parity tests."""
+import numpy as np
+import pytest
+
+from _gpu_helpers import compare_box, ctx_from, oracle_state_from_gpu, require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape,sc,threads", [(2, (8, 4, 4), 256), (2, (4, 4, 4), 64), (2, (8, 8, 8), 256),
+                                              (3, (8, 4, 4), 256), (1, (4, 4, 4), 128)])
+@pytest.mark.parametrize("n", [1, 255, 257, 1536, 1537, 3200])
+def test_sorted_lists(orc, n, shape, sc, threads):
+    require_gpu()
+    from paper_1606_02862_gb300 import workloads as W
+
+    rng = np.random.default_rng(100 + n)
+    N = 16
+    x = np.concatenate([8.0 + rng.random((n, 3)) * np.array([min(sc[0], 8), 4.0, 4.0]),
+                        rng.random((40, 3)) * N])
+    u = rng.normal(0, 0.1, x.shape)
+    w = 0.01 + 0.01 * rng.random(x.shape[0])
+    box = W.BoxInit(N, N, N, particles=[(x, u, w)], E=rng.normal(0, 1e-2, (3, N, N, N)), rho_bg=0.01)
+    wl = W.Workload("sort_test", W.DT_HALF_COURANT, [W.SpeciesDef("e", -1.0, 1.0, shape)], [box])
+    ctx = ctx_from(wl, sc=sc, threads_per_sc=threads, sort_every=1)
+    try:
+        ctx.step(3)
+        p = ctx.read_particles(0, 0, ids=True)
+        o = np.argsort(p["id"])
+        assert np.array_equal(p["id"][o], np.arange(x.shape[0]))
+        assert np.array_equal(p["w"][o], w.astype(np.float32).astype(np.float64))
+        st, ids = oracle_state_from_gpu(orc, ctx, wl, 0)
+        ctx.step(1)
+        st.step(1)
+        compare_box(st, ids, ctx, wl, 0, tol_field=1e-5, tol_x=1e-5, tol_u=1e-5)
+    finally:
+        ctx.close()
