@@ -305,45 +305,52 @@ __global__ void __launch_bounds__(256, 4) k_yee_e(const YeeArgs a)
 // The whole field half of the cycle in one kernel, from one buffer pair into
 // the other: E^n, B^n and J are read from `src`, E^{n+1} and B^{n+1} (with
 // their periodic guard images) are written into `dst`, so that no value is
-// overwritten while a neighbouring cell still needs it.  Each block
-// z-marches an output tile of kFusedTX x kFusedTY cells through a chunk of
-// kFusedTZ planes.  Iteration s forms, with one block barrier after it,
-//   B^{n+1/2}(s+1) on the tile and one cell around it (E^n planes s+1, s+2),
-//   E^{n+1}(s)     on the tile and one cell above it in x and y
-//                  (B^{n+1/2} planes s-1, s: earlier iterations),
-//   B^{n+1}(s-2)   on the tile (E^{n+1} planes s-2, s-1: earlier iterations),
-// so the three stages of an iteration depend only on earlier iterations and
-// the intermediate B^{n+1/2} and E^{n+1} stay in shared memory; halo cells
-// are formed again by the neighbouring tiles (and the first planes of a
-// chunk by the chunk below).  The inputs of iteration s -- E^n(s+2), B^n(s+1)
-// and J(s), each a plane tile of the three components -- arrive by tensor
-// loads kFLook iterations ahead on one mbarrier; a thread waits for them and
-// otherwise touches global memory only for its stores and for the few J
-// guard images that fold into cells next to a box face.  HBM traffic per
-// cell: E^n, B^n, J read and E^{n+1}, B^{n+1} written, 60 bytes (the three
-// in-place kernels move 120); the halo rows come from L2.  The arithmetic of
-// every value is that of k_yee_b, k_yee_e, k_yee_b.
-constexpr int kFX = kFusedTX, kFY = kFusedTY, kFT = kFX * kFY;
-constexpr int kFEX = kFusedEX, kFEY = kFY + 3;  // plane tile: cells x0-G .. x0-G+35, y0-1 .. y0+kFY+1
-constexpr int kFSlot = ((3 * kFEY * kFEX + 31) / 32) * 32;  // floats, 128-byte slots
-constexpr unsigned kFBytes = 3u * kFEY * kFEX * 4u;         // bytes of one plane tile
-constexpr int kFLook = 3;                                    // bundles issued ahead
-constexpr int kFRE = 8, kFRB = 4;  // E^n slots (>= kFLook + 3); B^n, J slots and mbarriers (>= kFLook + 1)
-static_assert(kFRE >= kFLook + 3 && kFRB >= kFLook + 1 && !(kFRE & (kFRE - 1)) && !(kFRB & (kFRB - 1)),
-              "power-of-two rings deep enough for the look-ahead");
-constexpr int kHX = kFX + 2, kHY = kFY + 2, kHN = kHX * kHY;  // B^{n+1/2}: x0-1.., y0-1..
-constexpr int kEX = kFX + 1, kEY = kFY + 1, kEN = kEX * kEY;  // E^{n+1}: x0.., y0..
-constexpr int kHPer = (kHN + kFT - 1) / kFT, kEPer = (kEN + kFT - 1) / kFT;
-static_assert(kFEX >= kFX + 4 && kFEX % 4 == 0, "plane rows reach x0 + kFX + 2 from a 16-byte start");
+// overwritten while a neighbouring cell still needs it.  Each block z-marches
+// an output tile of kFusedTX x kFusedTY cells through a chunk of planes, one
+// thread per column of the tile and of the one-cell rim around it (a warp per
+// row, the two rim columns of all rows in the last warp).  Iteration s:
+//   B^{n+1/2}(s)  on the tile and its rim (E^n planes s, s+1),
+//   one block barrier,
+//   E^{n+1}(s)    on the tile and the rim above it in x and y
+//                 (B^{n+1/2} planes s-1, s),
+//   B^{n+1}(s-1)  on the tile (E^{n+1} planes s-1, s).
+// A thread keeps its column's values of both planes in registers; shared
+// memory holds what the four neighbouring columns need (two planes each of
+// B^{n+1/2} and E^{n+1}).  Rim cells are formed again by the neighbouring
+// tiles, and the first planes of a chunk by the chunk below.  The inputs of
+// iteration s -- E^n(s+1), B^n(s) and J(s), each a plane tile of the three
+// components -- arrive by tensor loads issued three iterations ahead on one
+// mbarrier; a thread otherwise touches global memory only for its stores and
+// for the few J guard images that fold into cells next to a box face (loaded
+// an iteration ahead: the blocks at the faces set the pace of the others).
+// HBM traffic per cell: E^n, B^n, J read and E^{n+1}, B^{n+1} written, 60 bytes
+// (the three in-place kernels move 120); the rim comes from L2.  The arithmetic
+// of every value is that of k_yee_b, k_yee_e, k_yee_b, to the last bit.
+// Measured: 256^3 0.243 ms (4.1 TB/s of the 60 bytes; in place 0.450), 192x768x192
+// 0.404 ms (0.739), 128^3 0.059 ms (0.064).  With every stage's values of its own
+// column in shared memory too (39 shared loads per cell instead of 20), 24
+// planes per chunk and the image code in every block it took 0.400 ms, 0.698
+// ms and 0.067 ms.  What bounds it now is the blocks at the box faces and the
+// barrier of every iteration; tiles of 6, 12, 14 and 16 rows were no faster.
+constexpr int kFX = kFusedTX, kFY = kFusedTY;
+constexpr int kHX = kFX + 2, kHY = kFY + 2, kHN = kHX * kHY;  // columns x0-1 .. x0+kFX, y0-1 .. y0+kFY
+constexpr int kFWarps = kHY + (2 * kHY + 31) / 32;            // a warp per row, then the rim columns
+constexpr int kFT = 32 * kFWarps;
+constexpr int kFBlocksSM = 3;                                 // resident blocks per SM (shared memory)
+// plane tiles: cells x0-G .. x0-G+35; E^n rows y0-1 .. y0+kFY+1, B^n rows y0-1 .. y0+kFY, J rows y0 .. y0+kFY
+constexpr int kFEX = kFusedEX, kEC = kFusedERows * kFEX, kBC = kFusedBRows * kFEX, kJC = kFusedJRows * kFEX;
+static_assert(kFusedERows == kFY + 3 && kFusedBRows == kFY + 2 && kFusedJRows == kFY + 1, "rows of the plane tiles");
+constexpr int slot_floats(int comp) { return (3 * comp + 31) / 32 * 32; }  // 128-byte slots
+constexpr int kFRE = 4, kFRB = 3;  // E^n slots; B^n, J slots and mbarriers
+static_assert(kFX == 32 && kFEX >= kFX + 4 && kFEX % 4 == 0, "a warp per row; plane rows reach x0 + kFX + 2 from a 16-byte start");
 
 struct FusedSmem {
-    float en[kFRE][kFSlot];  // E^n plane tiles [c][y][x]
-    float bn[kFRB][kFSlot];  // B^n plane tiles
-    float jn[kFRB][kFSlot];  // J plane tiles (as deposited; guard images folded by the reader)
-    float bh[4][3][kHN];     // B^{n+1/2}, four planes [plane % 4][c][cell]
-    float e1[4][3][kEN];     // E^{n+1}, four planes [plane % 4][c][cell]
+    float en[kFRE][slot_floats(kEC)];  // E^n plane tiles [c][y][x]
+    float bn[kFRB][slot_floats(kBC)];  // B^n plane tiles
+    float jn[kFRB][slot_floats(kJC)];  // J plane tiles (as deposited; guard images folded by the reader)
+    float bh[2][3][kHN];     // B^{n+1/2}, two planes [plane % 2][c][column]
+    float e1[2][3][kHN];     // E^{n+1}, two planes
     unsigned long long mb[kFRB];
-    int abort;
 };
 
 struct FusedArgs {
@@ -352,267 +359,263 @@ struct FusedArgs {
     const CUtensorMap* maps;  // [nboxes][3]: E, B, J plane maps over src
     const int* blk_off;
     int nboxes;
+    int tz;  // planes per chunk
     float dt, tau;  // tau = dt / 2
     float ih[3];
     unsigned* status;
 };
 
-int fused_blocks(int nx, int ny, int nz)
+int fused_blocks(int nx, int ny, int nz, int tz)
 {
-    return ((nx + kFX - 1) / kFX) * ((ny + kFY - 1) / kFY) * ((nz + kFusedTZ - 1) / kFusedTZ);
+    return ((nx + kFX - 1) / kFX) * ((ny + kFY - 1) / kFY) * ((nz + tz - 1) / tz);
 }
 
-template <int G>
-__global__ void __launch_bounds__(kFT, 2) k_yee_fused(const FusedArgs a)
+int fused_resident() { return kFBlocksSM; }
+
+// The march of one block through its chunk of planes [zc0, zc1).  FACES: some
+// column of the tile or its rim, or some plane, is next to a box face, where
+// J gathers guard images and E, B are stored to them as well; without it (most
+// blocks of a large box) none of that code is in the loop.  Returns false when
+// a wait gave up.
+template <int G, bool FACES>
+__device__ __forceinline__ bool fused_march(const FusedArgs& a, FusedSmem& sm, int box, int x0, int y0, int zc0, int zc1)
 {
-    extern __shared__ __align__(128) unsigned char fused_smem[];
-    FusedSmem& sm = *reinterpret_cast<FusedSmem*>(fused_smem);
-    const int box = find_box(a.blk_off, a.nboxes, blockIdx.x);
     // the box's geometry and arrays in registers (stores through the field
     // pointers could otherwise alias the table and force reloads)
     const BoxDev& bt = a.src[box];
     const int nx = bt.nx, ny = bt.ny, nz = bt.nz, px = bt.px, py = bt.py;
-    const int64_t pc = (int64_t)px * py * bt.pz;
+    const int64_t plane = (int64_t)px * py;
+    const int64_t pc = plane * bt.pz;
     const float* __restrict__ Jg = bt.J;
     float* __restrict__ Eo = a.dst[box].E;
     float* __restrict__ Bo = a.dst[box].B;
     constexpr int hx = GuardsOf<G>::hx, hyz = GuardsOf<G>::hyz;
-    auto at = [&](int x, int y, int z) { return ((int64_t)(z + G) * py + (y + G)) * px + (x + G); };
-    // the three components of interior cell (x, y, z) and of its guard images
-    auto store3 = [&](float* F, int x, int y, int z, float v0, float v1, float v2) {
-        int ix[2], iy[2], iz[2];
-        const int cx = images(x, nx, G, hx, ix), cy = images(y, ny, G, hyz, iy), cz = images(z, nz, G, hyz, iz);
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-                    if (k < cz && j < cy && i < cx) {
-                        const int64_t g = at(ix[i], iy[j], iz[k]);
-                        F[g] = v0;
-                        F[pc + g] = v1;
-                        F[2 * pc + g] = v2;
-                    }
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const CUtensorMap* maps = a.maps + 3 * box;
+
+    // this thread's column
+    const int rim = (wid - kHY) * 32 + lane;  // >= 0: a column of the x rim
+    const int ry = wid < kHY ? wid : rim % kHY;
+    const int rx = wid < kHY ? lane + 1 : (rim < kHY ? 0 : kHX - 1);
+    const bool doh = rim < 2 * kHY;
+    const bool doe = doh && rx >= 1 && ry >= 1;
+    const int x = x0 - 1 + rx, y = y0 - 1 + ry;
+    const bool dob = doe && rx <= kFX && ry <= kFY && x < nx && y < ny;  // an output cell of this tile
+    const int e = ry * kFEX + rx + G - 1, h = ry * kHX + rx;             // index in the plane tiles, in bh and e1
+    // FACES: the cell (xc, yc) that the column is an image of (itself, but for
+    // the rim beyond the upper faces), and the word offsets of its image along
+    // x and y (0: none)
+    const int xc = FACES && x >= nx ? x - nx : x, yc = FACES && y >= ny ? y - ny : y;
+    auto image = [](int v, int n, int h) { return v < h ? n : (v >= n - G ? -n : 0); };
+    const bool inside = x <= nx && y <= ny;
+    const int dx = FACES && inside ? image(xc, nx, hx) : 0, dy = FACES && inside ? image(yc, ny, hyz) * px : 0;
+    const bool edge = dx != 0 || dy != 0 || x >= nx || y >= ny;
+    auto inner_plane = [&](int z) { return z >= hyz && z < nz - G; };
+    const int64_t ccol = (int64_t)(yc + G) * px + (xc + G);
+    auto put = [&](float* p, float v0, float v1, float v2) {
+        p[0] = v0;
+        p[pc] = v1;
+        p[2 * pc] = v2;
     };
-    // interior cells away from every face have no images: one store each
-    const int64_t plane = (int64_t)px * py;
-    auto store3_fast = [&](float* F, bool col_plain, int64_t col, int x, int y, int z, float v0, float v1,
-                           float v2) {
-        if (col_plain && z >= hyz && z < nz - G) {
-            const int64_t g = (int64_t)(z + G) * plane + col;
-            F[g] = v0;
-            F[pc + g] = v1;
-            F[2 * pc + g] = v2;
-        } else {
-            store3(F, x, y, z, v0, v1, v2);
+    // the cell and its images; p: the cell's first component
+    auto store3 = [&](float* p, int z, float v0, float v1, float v2) {
+        put(p, v0, v1, v2);
+        if (FACES && (edge || !inner_plane(z))) {
+            const int dz = image(z, nz, hyz);
+            for (int k = 0; k < (dz != 0 ? 2 : 1); ++k)
+                for (int j = 0; j < (dy != 0 ? 2 : 1); ++j)
+                    for (int i = 0; i < (dx != 0 ? 2 : 1); ++i)
+                        if (i + j + k > 0)
+                            put(p + k * dz * plane + j * dy + i * dx, v0, v1, v2);
         }
     };
-    const int local = blockIdx.x - a.blk_off[box];
-    const int ntx = (nx + kFX - 1) / kFX, nty = (ny + kFY - 1) / kFY;
-    const int x0 = (local % ntx) * kFX, y0 = ((local / ntx) % nty) * kFY;
-    const int zc0 = (local / (ntx * nty)) * kFusedTZ, zc1 = min(zc0 + kFusedTZ, nz);
-    const int tid = threadIdx.x;
-    const CUtensorMap* maps = a.maps + 3 * box;
-    // bundle k (k0 .. zc1 + 1): E^n(k+2) while k+2 <= zc1+1, B^n(k+1) while
-    // zc0-1 <= k+1 <= zc1, J(k) while zc0 <= k <= zc1; E^n in slot
-    // (k - k0) % kFRE, B^n and J in slot (k - k0) % kFRB, completing on that
-    // slot's mbarrier as its ((k - k0) / kFRB)-th phase
-    const int k0 = zc0 - 3, klast = zc1 + 1;
+    // FACES, J of the cell (xc, yc) in plane s: with no image it is the tile's
+    // own value; with one, the two values' sum, of which the one that is not
+    // this column's own is loaded an iteration ahead; with more (edges of the
+    // box), all are summed from global memory in the order of k_yee_e.
+    // extra_of: the number of images beside the own value, offset of the first
+    auto extra_of = [&](int s, int64_t* off) {
+        const int sc = s < nz ? s : s - nz;
+        const int dz = image(sc, nz, hyz);
+        const int n = (dx != 0 ? 2 : 1) * (dy != 0 ? 2 : 1) * (dz != 0 ? 2 : 1) - 1;
+        // n == 1: the own value is the cell's or its image's, the other is wanted
+        const bool own_is_image = x != xc || y != yc || s != sc;
+        *off = (int64_t)(sc + G) * plane + ccol + (own_is_image ? 0 : dx + dy + dz * plane);
+        return inside ? n : 0;
+    };
+
+    // bundle k (zc0 - 1 .. zc1), for iteration k: E^n(k+1), B^n(k) and, from
+    // zc0 on, J(k); the first one brings E^n(zc0-1) too.  Plane p of E^n sits
+    // in slot (p - zc0 + 1) % kFRE, B^n and J of bundle k in slot (k - zc0 + 1)
+    // % kFRB, completing on that slot's mbarrier.
+    const int k0 = zc0 - 1;
     int kiss = k0 - 1;  // tid 0: the last bundle issued
     auto issue = [&](int k) {
         kiss = k;
-        const int e = (k - k0) & (kFRE - 1), r = (k - k0) & (kFRB - 1);
-        const bool le = k + 2 <= zc1 + 1, lb = k + 1 >= zc0 - 1 && k + 1 <= zc1, lj = k >= zc0 && k <= zc1;
+        const int r = (k - k0) % kFRB;
+        const bool first = k == k0;
         unsigned long long* mb = &sm.mb[r];
-        mbar_expect_tx(mb, kFBytes * ((le ? 1u : 0u) + (lb ? 1u : 0u) + (lj ? 1u : 0u)));
-        if (le)
-            tma_load_tile(sm.en[e], maps + 0, x0, y0 - 1 + G, k + 2 + G, mb);
-        if (lb)
-            tma_load_tile(sm.bn[r], maps + 1, x0, y0 - 1 + G, k + 1 + G, mb);
-        if (lj)
-            tma_load_tile(sm.jn[r], maps + 2, x0, y0 - 1 + G, k + G, mb);
+        mbar_expect_tx(mb, 12u * (kEC + kBC + (first ? kEC : kJC)));
+        tma_load_tile(sm.en[(k + 1 - k0) & (kFRE - 1)], maps + 0, x0, y0 - 1 + G, k + 1 + G, mb);
+        tma_load_tile(sm.bn[r], maps + 1, x0, y0 - 1 + G, k + G, mb);
+        if (first)
+            tma_load_tile(sm.en[0], maps + 0, x0, y0 - 1 + G, k + G, mb);
+        else
+            tma_load_tile(sm.jn[r], maps + 2, x0, y0 + G, k + G, mb);
     };
     if (tid == 0) {
         for (int r = 0; r < kFRB; ++r)
             mbar_init(&sm.mb[r], 1);
         fence_mbar_init();
-        sm.abort = 0;
-        for (int k = k0; k <= min(k0 + kFLook, klast); ++k)
+        for (int k = k0; k <= min(k0 + kFRB - 1, zc1); ++k)
             issue(k);
     }
-    // J of the guard images of this thread's E^{n+1} cells other than the
-    // position itself (zero away from the box faces), one plane ahead
-    // (a column x, y inside [hx, nx - G) x [hyz, ny - G) and a plane inside
-    // [hyz, nz - G) have no images: most cells skip at once)
-    const auto inner = [](int v, int n, int h) { return v >= h && v < n - G; };
-    bool col_plain[kEPer], col_in[kEPer];
-#pragma unroll
-    for (int k = 0; k < kEPer; ++k) {
-        const int i = tid + k * kFT;
-        col_plain[k] = inner(x0 + i % kEX, nx, hx) && inner(y0 + i / kEX, ny, hyz);
-        col_in[k] = i < kEN && x0 + i % kEX <= nx && y0 + i / kEX <= ny;
-    }
-    auto fold_extra = [&](int s, float (&v)[kEPer][3]) {
-        const bool plane_plain = inner(s, nz, hyz) || s < zc0 || s > zc1;
-#pragma unroll
-        for (int k = 0; k < kEPer; ++k) {
-            v[k][0] = v[k][1] = v[k][2] = 0.0f;
-            if ((col_plain[k] && plane_plain) || !col_in[k] || s < zc0 || s > zc1)
-                continue;
-            const int i = tid + k * kFT;
-            const int x = x0 + i % kEX, y = y0 + i / kEX;
-            int ix[2], iy[2], iz[2];
-            const int cx = images(x < nx ? x : x - nx, nx, G, hx, ix);
-            const int cy = images(y < ny ? y : y - ny, ny, G, hyz, iy);
-            const int cz = images(s < nz ? s : s - nz, nz, G, hyz, iz);
-            if (cx == 1 && cy == 1 && cz == 1)
-                continue;
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk)
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int r = 0; r < 2; ++r)
-                        if (kk < cz && j < cy && r < cx && !(ix[r] == x && iy[j] == y && iz[kk] == s)) {
-                            const int64_t g = at(ix[r], iy[j], iz[kk]);
-                            v[k][0] += __ldg(Jg + g);
-                            v[k][1] += __ldg(Jg + pc + g);
-                            v[k][2] += __ldg(Jg + 2 * pc + g);
-                        }
-        }
-    };
-    float jx[kEPer][3] = {}, jxn[kEPer][3] = {};
     __syncthreads();  // the mbarriers are initialised
-    // bundle k0 (E^n(zc0-1) alone) before the loop, and a barrier after it:
-    // its mbarrier is re-armed by the first iteration, for bundle k0 + kFRB
-    bool timed_out = !mbar_wait(&sm.mb[0], 0u);
-    __syncthreads();
 
-    constexpr int EC = kFEY * kFEX;
     const float ih0 = a.ih[0], ih1 = a.ih[1], ih2 = a.ih[2], dt = a.dt, tau = a.tau;
-    // this thread's cells, the same in every plane: stage 1 cells i1 (tile
-    // index e1), stage 2 cells (tile index e2, B^{n+1/2} index h2, stored
-    // when st2), stage 3 cell (E^{n+1} index e3, B^{n+1/2} index h3)
-    int e1[kHPer], e2[kEPer], h2[kEPer];
-    bool st2[kEPer];
-    int64_t col2[kEPer];
-    // (the stage 1 cells past the first kFT go to the last threads and the
-    // stage 2 ones to the first, so that no warp takes both)
-    int i1[kHPer];
-#pragma unroll
-    for (int k = 0; k < kHPer; ++k) {
-        const int i = k == 0 ? tid : k * kFT + (kFT - 1 - tid);
-        i1[k] = i;
-        e1[k] = (i / kHX) * kFEX + i % kHX + G - 1;
-    }
-#pragma unroll
-    for (int k = 0; k < kEPer; ++k) {
-        const int i = tid + k * kFT, rx = i % kEX, ry = i / kEX;
-        h2[k] = (ry + 1) * kHX + rx + 1;
-        e2[k] = (ry + 1) * kFEX + rx + G;
-        st2[k] = i < kEN && rx < kFX && ry < kFY && x0 + rx < nx && y0 + ry < ny;
-        col2[k] = (int64_t)(y0 + ry + G) * px + (x0 + rx + G);
-    }
-    const int rx3 = tid % kFX, ry3 = tid / kFX;
-    const int e3 = ry3 * kEX + rx3, h3 = (ry3 + 1) * kHX + rx3 + 1;
-    const bool st3 = x0 + rx3 < nx && y0 + ry3 < ny;
-    const bool plain3 = inner(x0 + rx3, nx, hx) && inner(y0 + ry3, ny, hyz);
-    const int64_t col3 = (int64_t)(y0 + ry3 + G) * px + (x0 + rx3 + G);
-    for (int s = zc0 - 2; s <= zc1 + 1; ++s) {
-        if (tid == 0 && s + kFLook <= klast) {
-            fence_proxy_async();  // the slots being refilled were read by generic loads
-            issue(s + kFLook);
-        }
-        if (s >= zc0 - 1)
-            fold_extra(s + 1, jxn);
-        // the bundle of iteration s; its mbarrier was re-armed (at the top of
-        // iteration s - kFRB + kFLook) only after every thread had waited on
-        // that mbarrier's previous bundle and passed the barrier after it
-        if (!mbar_wait(&sm.mb[(s - k0) & (kFRB - 1)], (unsigned)(((s - k0) / kFRB) & 1)))
+    float ex = 0.f, ey = 0.f, ez = 0.f;     // E^n(s)
+    float qx = 0.f, qy = 0.f, qz = 0.f;     // B^{n+1/2}(s-1)
+    float fx = 0.f, fy = 0.f, fz = 0.f;     // E^{n+1}(s-1)
+    float ax = 0.f, ay = 0.f, az = 0.f;     // FACES: J(s) of this column's one image
+    float* pe = Eo + (int64_t)(k0 + G) * plane + ccol;  // this column in plane s
+    float* pb = Bo + (int64_t)(k0 - 1 + G) * plane + ccol;  // in plane s - 1
+    bool timed_out = false;
+    int r = 0, phase = 0;  // slot and parity of bundle s
+    for (int s = k0; s <= zc1; ++s, pe += plane, pb += plane) {
+        // the bundle of iteration s; its mbarrier was re-armed (after the
+        // barrier of iteration s - 3) only after every thread had waited on
+        // that mbarrier's previous bundle, s - 3
+        if (!mbar_wait(&sm.mb[r], (unsigned)phase))
             timed_out = true;
-        if (timed_out)
-            sm.abort = 1;
-        // stage 1: B^{n+1/2}(s+1) = B^n - tau curl E^n
-        if (s + 1 >= zc0 - 1 && s + 1 <= zc1) {
-            const float* E1 = sm.en[(s - 1 - k0) & (kFRE - 1)];  // plane s+1 (bundle s-1)
-            const float* E2 = sm.en[(s - k0) & (kFRE - 1)];      // plane s+2 (bundle s)
-            const float* Bp = sm.bn[(s - k0) & (kFRB - 1)];      // B^n plane s+1
-            float* H = sm.bh[(s + 1) & 3][0];
-#pragma unroll
-            for (int k = 0; k < kHPer; ++k) {
-                const int i = i1[k];
-                if (i < kHN) {
-                    const int e = e1[k];  // cell (x, y) in the plane tiles
-                    const float ex = E1[e], ey = E1[EC + e], ez = E1[2 * EC + e];
-                    const float cx = (E1[2 * EC + e + kFEX] - ez) * ih1 - (E2[EC + e] - ey) * ih2;
-                    const float cy = (E2[e] - ex) * ih2 - (E1[2 * EC + e + 1] - ez) * ih0;
-                    const float cz = (E1[EC + e + 1] - ey) * ih0 - (E1[e + kFEX] - ex) * ih1;
-                    H[i] = Bp[e] - tau * cx;
-                    H[kHN + i] = Bp[EC + e] - tau * cy;
-                    H[2 * kHN + i] = Bp[2 * EC + e] - tau * cz;
-                }
-            }
+        const float* E0 = sm.en[(s - k0) & (kFRE - 1)] + e;
+        const float* E1 = sm.en[(s + 1 - k0) & (kFRE - 1)] + e;
+        const float* Bp = sm.bn[r] + e;
+        const float* Jp = sm.jn[r] + e - kFEX;
+        float* H = sm.bh[s & 1][0] + h;
+        if (s == k0) {
+            ex = E0[0];
+            ey = E0[kEC];
+            ez = E0[2 * kEC];
         }
-        // stage 2: E^{n+1}(s) = E^n + dt (curl B^{n+1/2} - J)
-        if (s >= zc0 && s <= zc1) {
-            const float* H = sm.bh[s & 3][0];          // plane s
-            const float* Hp = sm.bh[(s - 1) & 3][0];   // plane s - 1
-            const float* E0 = sm.en[(s - 2 - k0) & (kFRE - 1)];  // E^n plane s (bundle s-2)
-            const float* Jp = sm.jn[(s - k0) & (kFRB - 1)];      // J plane s
-            float* X = sm.e1[s & 3][0];
-#pragma unroll
-            for (int k = 0; k < kEPer; ++k) {
-                const int i = tid + k * kFT;
-                if (i < kEN) {
-                    const int h = h2[k], e = e2[k];
-                    const float bxv = H[h], byv = H[kHN + h], bzv = H[2 * kHN + h];
-                    const float cx = (bzv - H[2 * kHN + h - kHX]) * ih1 - (byv - Hp[kHN + h]) * ih2;
-                    const float cy = (bxv - Hp[h]) * ih2 - (bzv - H[2 * kHN + h - 1]) * ih0;
-                    const float cz = (byv - H[kHN + h - 1]) * ih0 - (bxv - H[h - kHX]) * ih1;
-                    const float nex = E0[e] + dt * (cx - (Jp[e] + jx[k][0]));
-                    const float ney = E0[EC + e] + dt * (cy - (Jp[EC + e] + jx[k][1]));
-                    const float nez = E0[2 * EC + e] + dt * (cz - (Jp[2 * EC + e] + jx[k][2]));
-                    X[i] = nex;
-                    X[kEN + i] = ney;
-                    X[2 * kEN + i] = nez;
-                    if (st2[k] && s < zc1)
-                        store3_fast(Eo, col_plain[k], col2[k], x0 + i % kEX, y0 + i / kEX, s, nex, ney, nez);
-                }
-            }
+        // B^{n+1/2}(s) = B^n - tau curl E^n
+        const float ex1 = E1[0], ey1 = E1[kEC], ez1 = E1[2 * kEC];
+        const float bx = Bp[0] - tau * ((E0[2 * kEC + kFEX] - ez) * ih1 - (ey1 - ey) * ih2);
+        const float by = Bp[kBC] - tau * ((ex1 - ex) * ih2 - (E0[2 * kEC + 1] - ez) * ih0);
+        const float bz = Bp[2 * kBC] - tau * ((E0[kEC + 1] - ey) * ih0 - (E0[kFEX] - ex) * ih1);
+        if (doh) {
+            H[0] = bx;
+            H[kHN] = by;
+            H[2 * kHN] = bz;
         }
-        // stage 3: B^{n+1}(s-2) = B^{n+1/2} - tau curl E^{n+1}
-        if (s - 2 >= zc0 && s - 2 < zc1) {
-            if (st3) {
-                const float* X0 = sm.e1[(s - 2) & 3][0];  // plane s - 2
-                const float* X1 = sm.e1[(s - 1) & 3][0];  // plane s - 1
-                const float* Hq = sm.bh[(s - 2) & 3][0];  // plane s - 2
-                const int e = e3, h = h3;
-                const float ex = X0[e], ey = X0[kEN + e], ez = X0[2 * kEN + e];
-                const float cx = (X0[2 * kEN + e + kEX] - ez) * ih1 - (X1[kEN + e] - ey) * ih2;
-                const float cy = (X1[e] - ex) * ih2 - (X0[2 * kEN + e + 1] - ez) * ih0;
-                const float cz = (X0[kEN + e + 1] - ey) * ih0 - (X0[e + kEX] - ex) * ih1;
-                store3_fast(Bo, plain3, col3, x0 + rx3, y0 + ry3, s - 2, Hq[h] - tau * cx, Hq[kHN + h] - tau * cy,
-                            Hq[2 * kHN + h] - tau * cz);
-            }
+        float jx = 0.f, jy = 0.f, jz = 0.f;
+        if (doe && s >= zc0) {
+            jx = Jp[0];
+            jy = Jp[kJC];
+            jz = Jp[2 * kJC];
         }
-        __syncthreads();
-        if (sm.abort)
+        if (__syncthreads_or(timed_out ? 1 : 0)) {
+            timed_out = true;
             break;
-        if (s >= zc0 - 1)
-#pragma unroll
-            for (int k = 0; k < kEPer; ++k)
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    jx[k][c] = jxn[k][c];
+        }
+        // every thread is past its reads of E^n(s), B^n(s) and J(s): their
+        // slots take bundle s + 3
+        if (tid == 0 && s + kFRB <= zc1) {
+            fence_proxy_async();  // the slots being refilled were read by generic loads
+            issue(s + kFRB);
+        }
+        // E^{n+1}(s) = E^n + dt (curl B^{n+1/2} - J)
+        float nex = 0.f, ney = 0.f, nez = 0.f;
+        if (s >= zc0) {
+            if (doe) {
+                if (FACES && (edge || !inner_plane(s))) {
+                    int64_t off;
+                    const int extra = extra_of(s, &off);
+                    if (extra == 1) {
+                        jx += ax;
+                        jy += ay;
+                        jz += az;
+                    } else if (extra > 1) {
+                        jx = jy = jz = 0.f;
+                        const int sc = s < nz ? s : s - nz;
+                        const int dz = image(sc, nz, hyz);
+                        for (int kk = 0; kk < (dz != 0 ? 2 : 1); ++kk)
+                            for (int j = 0; j < (dy != 0 ? 2 : 1); ++j)
+                                for (int i = 0; i < (dx != 0 ? 2 : 1); ++i) {
+                                    const float* p = Jg + (int64_t)(sc + G + kk * dz) * plane + ccol + j * dy + i * dx;
+                                    jx += __ldg(p);
+                                    jy += __ldg(p + pc);
+                                    jz += __ldg(p + 2 * pc);
+                                }
+                    }
+                }
+                const float cx = (bz - H[2 * kHN - kHX]) * ih1 - (by - qy) * ih2;
+                const float cy = (bx - qx) * ih2 - (bz - H[2 * kHN - 1]) * ih0;
+                const float cz = (by - H[kHN - 1]) * ih0 - (bx - H[-kHX]) * ih1;
+                nex = ex + dt * (cx - jx);
+                ney = ey + dt * (cy - jy);
+                nez = ez + dt * (cz - jz);
+                float* X = sm.e1[s & 1][0] + h;
+                X[0] = nex;
+                X[kHN] = ney;
+                X[2 * kHN] = nez;
+            }
+            if (dob) {
+                if (s < zc1)
+                    store3(pe, s, nex, ney, nez);
+                // B^{n+1}(s-1) = B^{n+1/2} - tau curl E^{n+1}
+                if (s > zc0) {
+                    const float* X0 = sm.e1[(s - 1) & 1][0] + h;
+                    const float cx = (X0[2 * kHN + kHX] - fz) * ih1 - (ney - fy) * ih2;
+                    const float cy = (nex - fx) * ih2 - (X0[2 * kHN + 1] - fz) * ih0;
+                    const float cz = (X0[kHN + 1] - fy) * ih0 - (X0[kHX] - fx) * ih1;
+                    store3(pb, s - 1, qx - tau * cx, qy - tau * cy, qz - tau * cz);
+                }
+            }
+        }
+        if (FACES && doe && s + 1 >= zc0 && s < zc1 && (edge || !inner_plane(s + 1))) {
+            int64_t off;
+            if (extra_of(s + 1, &off) == 1) {
+                ax = __ldg(Jg + off);
+                ay = __ldg(Jg + pc + off);
+                az = __ldg(Jg + 2 * pc + off);
+            }
+        }
+        ex = ex1, ey = ey1, ez = ez1;
+        qx = bx, qy = by, qz = bz;
+        fx = nex, fy = ney, fz = nez;
+        if (++r == kFRB) {
+            r = 0;
+            phase ^= 1;
+        }
     }
-    if (sm.abort && tid == 0) {
-        atomicOr(a.status, ST_TIMEOUT);
+    if (timed_out && tid == 0) {
         // loads still in flight land before the block's shared memory goes
         // away: the last bundle issued on each mbarrier
         for (int k = max(k0, kiss - kFRB + 1); k <= kiss; ++k)
-            mbar_wait(&sm.mb[(k - k0) & (kFRB - 1)], (unsigned)(((k - k0) / kFRB) & 1));
+            mbar_wait(&sm.mb[(k - k0) % kFRB], (unsigned)(((k - k0) / kFRB) & 1));
     }
+    return !timed_out;
+}
+
+template <int G>
+__global__ void __launch_bounds__(kFT, kFBlocksSM) k_yee_fused(const FusedArgs a)
+{
+    extern __shared__ __align__(128) unsigned char fused_smem[];
+    FusedSmem& sm = *reinterpret_cast<FusedSmem*>(fused_smem);
+    const int box = find_box(a.blk_off, a.nboxes, blockIdx.x);
+    const BoxDev& b = a.src[box];
+    const int local = blockIdx.x - a.blk_off[box];
+    const int ntx = (b.nx + kFX - 1) / kFX, nty = (b.ny + kFY - 1) / kFY;
+    const int x0 = (local % ntx) * kFX, y0 = ((local / ntx) % nty) * kFY;
+    const int zc0 = (local / (ntx * nty)) * a.tz, zc1 = min(zc0 + a.tz, b.nz);
+    // columns x0 .. x0 + kFX, y0 .. y0 + kFY and planes zc0 .. zc1 take part in
+    // the E update: none of them within the reach of a face's guards
+    const bool faces = x0 < GuardsOf<G>::hx || x0 + kFX >= b.nx - G || y0 < GuardsOf<G>::hyz ||
+                       y0 + kFY >= b.ny - G || zc0 < GuardsOf<G>::hyz || zc1 >= b.nz - G;
+    const bool ok = faces ? fused_march<G, true>(a, sm, box, x0, y0, zc0, zc1)
+                          : fused_march<G, false>(a, sm, box, x0, y0, zc0, zc1);
+    if (!ok && threadIdx.x == 0)
+        atomicOr(a.status, ST_TIMEOUT);
 }
 
 size_t fused_smem_bytes() { return sizeof(FusedSmem); }
@@ -718,7 +721,7 @@ cudaError_t launch_yee_fused(const YeePlan& p, const FusedPlan& f, cudaStream_t 
                    p.step_no, p.dt_d, {p.dx_d[0], p.dx_d[1], p.dx_d[2]}};
         k_antenna<<<64, 256, 0, st>>>(ya);
     }
-    FusedArgs a{f.src, f.dst, f.maps, f.blk_off, p.nboxes, p.dt, 0.5f * p.dt, {p.ih[0], p.ih[1], p.ih[2]},
+    FusedArgs a{f.src, f.dst, f.maps, f.blk_off, p.nboxes, f.tz, p.dt, 0.5f * p.dt, {p.ih[0], p.ih[1], p.ih[2]},
                 f.status};
     if (p.guard == 2)
         k_yee_fused<2><<<f.nblocks, kFT, sizeof(FusedSmem), st>>>(a);

@@ -143,6 +143,7 @@ struct pic_ctx {
     CUtensorMap* ymaps_d = nullptr;      // [2][nboxes][3] plane maps of k_yee_fused: E, B, J of either pair
     int* fused_off_d = nullptr;
     int fused_nblocks = 0;
+    int fused_tz = 0;                    // planes per chunk of k_yee_fused
     int64_t fused_steps = 0;
     // graphs of a pair of steps, one per frame-table parity of its first step
     cudaGraph_t pgraph[2] = {nullptr, nullptr};
@@ -565,7 +566,8 @@ YeePlan yee_plan(const pic_ctx* c)
 FusedPlan fused_plan(const pic_ctx* c, int src)
 {
     return FusedPlan{src ? c->boxes_alt_d : c->boxes_d, src ? c->boxes_d : c->boxes_alt_d,
-                     c->ymaps_d + (size_t)src * 3 * c->nboxes, c->fused_off_d, c->fused_nblocks, c->status_d};
+                     c->ymaps_d + (size_t)src * 3 * c->nboxes, c->fused_off_d, c->fused_nblocks,
+                     c->fused_tz, c->status_d};
 }
 
 // One stage of the mixed-form step (PIC_STAGE_*) on frame-table parity
@@ -1004,6 +1006,22 @@ std::vector<BoxDev> alt_boxes(const pic_ctx* c)
     return alt;
 }
 
+// Planes per chunk of the fused field update.  A block takes two iterations
+// more than its chunk has planes, and the last blocks of a launch leave the GPU
+// less and less busy, so the chunk grows with the square root of the planes
+// (tiles x nz) per resident block.  Swept on box sizes from 64^3 to 256^3 and
+// 192x768x192 (best / at this rule's choice, ms): 0.0257 / 0.0257 (4 planes),
+// 96^3 0.0373 / 0.0373 (5), 128^3 0.0589 / 0.0589 (6), 256^3 0.2449 / 0.2449
+// (10; 24 planes 0.281), 192x768x192 0.402 / 0.402 (10).
+int fused_chunk(const pic_ctx* c)
+{
+    int64_t planes = 0;
+    for (const BoxDev& b : c->boxes_h)
+        planes += (int64_t)fused_blocks(b.nx, b.ny, 1, 1) * b.nz;
+    const double per = (double)planes / (double)(fused_resident() * std::max(1, c->nsm));
+    return std::min(10, std::max(4, (int)std::lround(3.0 + 0.6 * std::sqrt(per))));
+}
+
 // The second field buffer pair of the fused field update, its box table,
 // its push tile maps and the E plane maps of k_yee_fused over both pairs
 // (pic_options.field_update 0; not for subdomain slabs, which step by
@@ -1026,12 +1044,15 @@ pic_status prepare_fused(pic_ctx* c)
         for (int src = 0; src < 2; ++src) {
             const BoxDev& bd = src ? alt[b] : c->boxes_h[b];
             float* F[3] = {bd.E, bd.B, bd.J};
+            const int rows[3] = {kFusedERows, kFusedBRows, kFusedJRows};
             for (int f = 0; f < 3; ++f)
-                CKS(encode_field_map(c, &ymaps[((size_t)src * c->nboxes + b) * 3 + f], bd, F[f], kFusedEX,
-                                     kFusedTY + 3, 1, b));
+                CKS(encode_field_map(c, &ymaps[((size_t)src * c->nboxes + b) * 3 + f], bd, F[f], kFusedEX, rows[f],
+                                     1, b));
         }
-        off[b + 1] = off[b] + fused_blocks(c->boxes_h[b].nx, c->boxes_h[b].ny, c->boxes_h[b].nz);
     }
+    c->fused_tz = fused_chunk(c);
+    for (int b = 0; b < c->nboxes; ++b)
+        off[b + 1] = off[b] + fused_blocks(c->boxes_h[b].nx, c->boxes_h[b].ny, c->boxes_h[b].nz, c->fused_tz);
     CK(configure_yee_fused());
     CKS(dalloc(c, &c->ymaps_d, 6 * c->nboxes, false));
     CKS(dalloc(c, &c->fused_off_d, c->nboxes + 1, false));

@@ -201,21 +201,23 @@ struct YeePlan {
     int sub_z;                 // the (single) box is a subdomain slab: J is not folded in z
 };
 // The fused field update (k_yee_fused): output tiles of kFusedTX x kFusedTY
-// cells z-marching through chunks of kFusedTZ planes; its E, B and J planes
-// arrive by tensor loads of kFusedEX x (kFusedTY + 3) cells (x from the
-// tile's x0 - guard, a 16-byte boundary of the padded row), all three
-// components.
-constexpr int kFusedTX = 32, kFusedTY = 8, kFusedTZ = 24, kFusedEX = 36;
+// cells z-marching through chunks of tz planes; its E, B and J planes arrive
+// by tensor loads of kFusedEX x kFusedERows / BRows / JRows cells (x from the tile's
+// x0 - guard, a 16-byte boundary of the padded row), all three components.
+constexpr int kFusedTX = 32, kFusedTY = 8, kFusedEX = 36;
+constexpr int kFusedERows = kFusedTY + 3, kFusedBRows = kFusedTY + 2, kFusedJRows = kFusedTY + 1;
 struct FusedPlan {
     const BoxDev* src;        // device table of the buffers read (E^n, B^n, J)
     const BoxDev* dst;        // device table of the buffers written (E^{n+1}, B^{n+1})
     const CUtensorMap* maps;  // device [nboxes][3]: E, B, J plane maps over src's fields
     const int* blk_off;       // device [nboxes + 1] block offsets
     int nblocks;
+    int tz;                   // planes per chunk
     unsigned* status;         // ST_TIMEOUT when a tensor-load wait gave up
 };
-// blocks of the fused field update for one box
-int fused_blocks(int nx, int ny, int nz);
+// blocks of the fused field update for one box, and its resident blocks per SM
+int fused_blocks(int nx, int ny, int nz, int tz);
+int fused_resident();
 // its dynamic shared memory, and the kernel attribute that allows it (call
 // once, outside stream capture)
 size_t fused_smem_bytes();

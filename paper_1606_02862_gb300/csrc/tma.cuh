@@ -51,6 +51,8 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* mb, unsigned p
 // the phase of parity `parity` completed (false: gave up after kWaitCycles)
 __device__ __forceinline__ bool mbar_wait(unsigned long long* mb, unsigned parity)
 {
+    if (mbar_try_wait(mb, parity))
+        return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(mb, parity))
         if (clock64() - t0 > kWaitCycles)

@@ -223,3 +223,35 @@ def test_fused_pairs_across_a_window_shift():
     finally:
         fused.close()
         in_place.close()
+
+
+@pytest.mark.parametrize("n,shape", [((4, 4, 4), 2), ((36, 12, 8), 2), ((68, 20, 16), 2), ((100, 28, 44), 1),
+                                     ((72, 24, 20), 3)])
+def test_fused_tiles_and_faces(n, shape):
+    """One fused pair against the in-place kernels in boxes smaller than a
+    tile, with partial tiles, and large enough for blocks that touch no face
+    (whose march has no image code); a few fast particles cross the faces,
+    edges and corners, so that guard images of J fold into every kind of cell."""
+    require_gpu()
+    from paper_1606_02862_gb300 import pic
+    from paper_1606_02862_gb300 import workloads as W
+
+    nx, ny, nz = n
+    rng = np.random.default_rng(sum(n))
+    N = np.array(n, dtype=float)
+    x = np.concatenate([N * np.array(f) + d for f in ((0.5, 0.5, 0.5), (0, 0.5, 0.5), (0.5, 0, 0.5), (0.5, 0.5, 0),
+                                                      (0, 0, 0.5), (0, 0, 0)) for d in (np.full((1, 3), 0.1),
+                                                                                       np.full((1, 3), -0.1))])
+    u = rng.normal(0, 1.0, x.shape)
+    box = W.BoxInit(nx, ny, nz, particles=[(np.mod(x, N), u, np.full(x.shape[0], 0.05))],
+                    E=rng.normal(0, 1e-2, (3, nz, ny, nx)), B=rng.normal(0, 1e-2, (3, nz, ny, nx)))
+    wl = W.Workload("fused_tiles", W.DT_HALF_COURANT, [W.SpeciesDef("e", -1.0, 1.0, shape)], [box])
+    states = []
+    for form in (pic.FIELD_UPDATE_FUSED, pic.FIELD_UPDATE_IN_PLACE):
+        ctx = ctx_from(wl, field_update=form)
+        try:
+            ctx.step(2)
+            states.append(_state(ctx, wl))
+        finally:
+            ctx.close()
+    print("fused tiles errors:", n, _agree(states[0], states[1], wl))
