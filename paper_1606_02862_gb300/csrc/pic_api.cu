@@ -2128,6 +2128,12 @@ pic_status pic_read_fields(pic_ctx* c, int32_t box, int32_t which, double* out)
         return fail(c, PIC_ERR_ARG, "bad arguments to pic_read_fields");
     const pic_grid& g = c->grids[box];
     const int64_t nc = (int64_t)g.nx * g.ny * g.nz;
+    if (which == PIC_FIELD_RHO && c->precision == PIC_PRECISION_MIXED) {
+        CK(launch_rho_mixed(make_step(c, c->parity), c->boxes_h[box], box, c->rho_bg[box], c->rho_d, c->h, c->stream));
+        CK(cudaMemcpyAsync(out, c->rho_d, sizeof(double) * nc, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        return PIC_OK;
+    }
     if (which == PIC_FIELD_RHO) {
         double tmp[4];
         CKS(pic_diagnostics(c, box, tmp));

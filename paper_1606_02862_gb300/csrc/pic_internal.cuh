@@ -269,4 +269,7 @@ cudaError_t launch_fields_from_padded(const BoxDev& b, int which, double* dst, c
 cudaError_t launch_diag_mixed(const StepDev& d, const BoxDev& hb, int box, double rho_bg,
                               double* rho_scratch, double* out, const double h[3],
                               cudaStream_t st);
+// the charge density of the box at the nodes, background included
+cudaError_t launch_rho_mixed(const StepDev& d, const BoxDev& hb, int box, double rho_bg, double* rho,
+                             const double h[3], cudaStream_t st);
 }  // namespace pic
