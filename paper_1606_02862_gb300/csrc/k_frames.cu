@@ -6,7 +6,7 @@
 // and holds count[L] particles; narrive[L] particles from neighbouring
 // supercells wait in the move buffer, each with its rank among the arrivals
 // of its destination list.  One step of maintenance:
-//   scan_reduce / scan_top / scan_apply: an exclusive prefix sum over the
+//   scan_reduce / scan_top / scan_apply (few lists: scan_small alone): an exclusive prefix sum over the
 //     lists of (frames needed, frames to allocate, frames to release) gives
 //     every list its place in the next frame table; scan_apply also copies
 //     the kept frame indices, pops new frames off the free stack and queues
@@ -129,28 +129,37 @@ __global__ void __launch_bounds__(1024) k_scan_top(const StepDev d, int nblk)
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const StepDev d)
+// Whether the pool holds the frames that the plan `tot` needs; says so in the
+// status word if not (the step's arrivals are abandoned).
+__device__ __forceinline__ bool pool_holds(const StepDev& d, int4 tot)
 {
-    const int4 tot = *d.totals;
-    const int top = *d.free_top;
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *d.nitems = 0;  // k_place counts them anew
-    if (tot.y > top) {
-        // pool exhausted: report it; the step's arrivals are abandoned
-        if (blockIdx.x == 0 && threadIdx.x == 0)
-            atomicOr(d.status, ST_FRAME_POOL);
-        return;
-    }
-    const int alloc_base = top - tot.y;
-    const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-    int4 need[kScanItems];
+    if (tot.y <= *d.free_top)
+        return true;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        atomicOr(d.status, ST_FRAME_POOL);
+    return false;
+}
+
+// This thread's kScanItems lists from `base` on: what each needs, and the sum.
+__device__ __forceinline__ int4 lists_need(const StepDev& d, int base, int4 (&need)[kScanItems])
+{
     int4 acc = make_int4(0, 0, 0, 0);
     for (int i = 0; i < kScanItems; ++i) {
-        int L = base + i;
+        const int L = base + i;
         need[i] = L < d.nlists ? list_need(d, L) : make_int4(0, 0, 0, 0);
         acc = acc + need[i];
     }
-    int4 off = block_exclusive_scan<kScanThreads>(acc, nullptr) + d.blk_offs[blockIdx.x];
+    return acc;
+}
+
+// Writes this thread's lists into the next frame table, `off` being the
+// prefix sum over the lists before them.
+__device__ __forceinline__ void apply_lists(const StepDev& d, int4 tot, int base, int4 off,
+                                            const int4 (&need)[kScanItems])
+{
+    const int alloc_base = *d.free_top - tot.y;
     for (int i = 0; i < kScanItems; ++i) {
         int L = base + i;
         if (L >= d.nlists)
@@ -174,6 +183,35 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const StepDev d)
         d.narrive[L] = 0;
         off = off + need[i];
     }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const StepDev d)
+{
+    const int4 tot = *d.totals;
+    if (!pool_holds(d, tot))
+        return;
+    const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
+    int4 need[kScanItems];
+    const int4 acc = lists_need(d, base, need);
+    apply_lists(d, tot, base, block_exclusive_scan<kScanThreads>(acc, nullptr) + d.blk_offs[blockIdx.x], need);
+}
+
+// k_scan_reduce, k_scan_top and k_scan_apply in one block, for at most
+// kScanTile lists: a small step is a row of launches of a few microseconds each
+// (32^3 CIC, 512 lists: 22.9 us for the five kernels of the maintenance).
+__global__ void __launch_bounds__(kScanThreads) k_scan_small(const StepDev d)
+{
+    const int base = threadIdx.x * kScanItems;
+    int4 need[kScanItems], tot;
+    const int4 acc = lists_need(d, base, need);
+    const int4 off = block_exclusive_scan<kScanThreads>(acc, &tot);
+    if (threadIdx.x == 0) {
+        *d.totals = tot;
+        ++*d.step_ctr;
+        ++*d.step_no;
+    }
+    if (pool_holds(d, tot))
+        apply_lists(d, tot, base, off, need);
 }
 
 // The work items of the next push: the supercells with a particle of a
@@ -412,6 +450,7 @@ __global__ void __launch_bounds__(kSortThreads) k_finish(const StepDev d)
                 *d.free_top = top - tot.y + tot.z;
                 *d.mv_count = 0;
             }
+            *d.work_counter = 0;  // of the next push
         }
         return;
     }
@@ -484,6 +523,8 @@ cudaError_t launch_rotate_lists(const StepDev& d, const BoxDev& hb, const int* o
     return cudaGetLastError();
 }
 
+int frame_launches(int nlists) { return nlists > kScanTile ? 5 : 3; }
+
 int frame_scan_blocks(int nlists) { return (nlists + kScanTile - 1) / kScanTile; }
 
 cudaError_t launch_frame_plan(const StepDev& d, cudaStream_t st)
@@ -494,13 +535,28 @@ cudaError_t launch_frame_plan(const StepDev& d, cudaStream_t st)
     return cudaGetLastError();
 }
 
+static cudaError_t launch_placing(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st)
+{
+    k_place<<<place_blocks, 256, 0, st>>>(d);
+    k_finish<<<1 + sort_blocks, kSortThreads, sort_blocks > 0 ? sort_smem_bytes(d.pid != nullptr) : 0, st>>>(d);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_frame_apply(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st)
 {
     const int nblk = frame_scan_blocks(d.nlists);
     k_scan_apply<<<nblk, kScanThreads, 0, st>>>(d);
-    k_place<<<place_blocks, 256, 0, st>>>(d);
-    k_finish<<<1 + sort_blocks, kSortThreads, sort_blocks > 0 ? sort_smem_bytes(d.pid != nullptr) : 0, st>>>(d);
-    return cudaGetLastError();
+    return launch_placing(d, place_blocks, sort_blocks, st);
+}
+
+cudaError_t launch_frames(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st)
+{
+    if (d.nlists > kScanTile) {
+        const cudaError_t e = launch_frame_plan(d, st);
+        return e != cudaSuccess ? e : launch_frame_apply(d, place_blocks, sort_blocks, st);
+    }
+    k_scan_small<<<1, kScanThreads, 0, st>>>(d);
+    return launch_placing(d, place_blocks, sort_blocks, st);
 }
 
 // ------------------------------------------------------------ subdomain migrants

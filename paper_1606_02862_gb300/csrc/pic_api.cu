@@ -570,6 +570,23 @@ FusedPlan fused_plan(const pic_ctx* c, int src)
                      c->fused_tz, c->status_d};
 }
 
+// Blocks of the kernels that end the frame maintenance: 4 per SM, or what a
+// small context can occupy (an eighth of its particles moving, a thread per
+// supercell); none for the sort where no species' lists are sorted there.
+int place_blocks(const pic_ctx* c)
+{
+    const int64_t threads = std::max<int64_t>(c->total_particles / 8, c->nsc);
+    return (int)std::min<int64_t>(4 * c->nsm, threads / 256 + 1);
+}
+
+int sort_blocks(const pic_ctx* c)
+{
+    for (const pic_species& p : c->sp)
+        if (p.mobile && p.shape != 1)
+            return std::min(4 * c->nsm, c->nlists);
+    return 0;
+}
+
 // One stage of the mixed-form step (PIC_STAGE_*) on frame-table parity
 // `parity`; the Yee stages run one part of the field update each.  fsrc 0 /
 // 1: a step of a fused pair, whose fields are read from the first / second
@@ -580,7 +597,7 @@ pic_status enqueue_stage(pic_ctx* c, int stage, int parity, int fsrc = -1)
     const StepDev d = make_step(c, parity, fsrc == 1);
     switch (stage) {
     case PIC_STAGE_PUSH:
-        CK(cudaMemsetAsync(c->work_counter, 0, sizeof(int), c->stream));
+        // (the work counter: zeroed by the frame maintenance before)
         CK(cudaMemsetAsync(c->J_all, 0, sizeof(float) * c->field_floats, c->stream));
         if (c->mig) {  // the face messages start empty (their capacity word stays)
             CK(cudaMemsetAsync(c->mig, 0, sizeof(int), c->stream));
@@ -589,8 +606,7 @@ pic_status enqueue_stage(pic_ctx* c, int stage, int parity, int fsrc = -1)
         CK(launch_push_deposit(d, c->threads, c->push_grid, c->stream));
         return PIC_OK;
     case PIC_STAGE_FRAMES:
-        CK(launch_frame_plan(d, c->stream));
-        CK(launch_frame_apply(d, 4 * c->nsm, 4 * c->nsm, c->stream));
+        CK(launch_frames(d, place_blocks(c), sort_blocks(c), c->stream));
         return PIC_OK;
     default:
         CK(launch_yee_mixed_part(yee_plan(c), stage - PIC_STAGE_B_FIRST, c->stream));
@@ -2196,12 +2212,12 @@ pic_status pic_info(pic_ctx* c, int32_t key, int64_t* out)
         return PIC_OK;
     case PIC_INFO_KERNELS_PER_STEP:
         if (c->precision == PIC_PRECISION_MIXED) {
-            // push; scan reduce, top; apply, place, free; Yee x3; antenna; y absorber;
+            // push; frame maintenance; Yee x3; antenna; y absorber;
             // a subdomain slab adds its 16 halo pack/unpack launches (J, B, E, B:
             // two faces each way) and 2 migrant accepts
             // (the fused field update: one kernel for the three)
             const bool fused = c->fused_ready;
-            *out = 1 + 2 + 3 + (fused ? 1 : 3) + (c->any_antenna ? 1 : 0) + (c->abs_nblocks > 0 ? 1 : 0) +
+            *out = 1 + frame_launches(c->nlists) + (fused ? 1 : 3) + (c->any_antenna ? 1 : 0) + (c->abs_nblocks > 0 ? 1 : 0) +
                    (c->sub_z ? 18 : 0);
         } else {
             int64_t k = 0;

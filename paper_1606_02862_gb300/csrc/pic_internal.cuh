@@ -236,6 +236,10 @@ cudaError_t launch_frame_plan(const StepDev& d, cudaStream_t st);
 // sort_blocks > 0: blocks that sort the lists when the step count says so
 // (d.step_ctr; configure_sort called before)
 cudaError_t launch_frame_apply(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st);
+// both, for a step
+cudaError_t launch_frames(const StepDev& d, int place_blocks, int sort_blocks, cudaStream_t st);
+// the launches of launch_frames for nlists lists
+int frame_launches(int nlists);
 // the sort's shared-memory limit (call once, outside stream capture), and a
 // sort of every list now
 cudaError_t configure_sort();
