@@ -42,7 +42,7 @@ MIXED_BYTES_PER_CELL = 36.0
 # plain FP64 form: particle read 56 B + write 48 B; fields 48 + 24 B/cell
 PLAIN_BYTES_PER_PARTICLE = 104.0
 PLAIN_BYTES_PER_CELL = 72.0
-PUSH_KERNEL_SRC = os.path.join(ROOT, "paper_1606_02862_gb300", "csrc", "k_push.cu")
+PUSH_KERNEL_SRC = os.path.join(ROOT, "paper_1606_02862_gb300", "csrc", "k_push.cuh")
 # machine-readable figures of the committed ncu summary of the push kernel
 TRAFFIC_SUMMARY = os.path.join(ROOT, "profiles", "push_deposit_thermal_tsc.json")
 

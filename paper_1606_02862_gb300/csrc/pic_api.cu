@@ -72,6 +72,7 @@ struct pic_ctx {
     int LX = 4, LY = 4, LZ = 4, S = 64, log2S = 6, threads = 64;
     int guard = 1;  // field guard cells below the interior: 2 when a species has the PCS shape
     int push_grid = 0;
+    int push_only = 0;  // StepDev::push_only
     std::vector<BoxDev> boxes_h;
     BoxDev* boxes_d = nullptr;
     CUtensorMap* tmaps_d = nullptr;  // [nboxes][2] E, B tile maps of the push
@@ -383,6 +384,7 @@ StepDev make_step(const pic_ctx* c, int parity, bool alt = false)
     d.nsc = c->nsc;
     d.nspecies = (int)c->sp.size();
     d.nlists = c->nlists;
+    d.push_only = c->push_only;
     d.dt = (float)c->dt;
     for (int a = 0; a < 3; ++a)
         d.move[a] = (float)(c->dt / c->h[a]);
@@ -663,7 +665,7 @@ pic_status prepare_mixed(pic_ctx* c)
                                           : std::max<int64_t>(1 << 20, c->total_particles / 6);
     CKS(ensure_mv(c, mv));
     int per_sm = 0;
-    CK(configure_push(c->LX, c->LY, c->LZ, c->threads, c->guard, &per_sm));
+    CK(configure_push(c->LX, c->LY, c->LZ, c->threads, c->guard, c->push_only, &per_sm));
     c->push_grid = std::max(1, per_sm) * c->nsm;
     // freshly loaded particles sit unsorted at the ends of their lists
     CK(configure_sort());
@@ -1281,6 +1283,15 @@ pic_status pic_create(const pic_grid* grids, int32_t nboxes, const double dx[3],
         for (int s = 0; s < nspecies; ++s)
             if (sp[s].shape == 3)
                 c->guard = 2;
+        // the push kernel with one shape's code alone: fewer registers and less
+        // shared memory than the one for any mix
+        c->push_only = -1;
+        for (int s = 0; s < nspecies; ++s)
+            if (sp[s].mobile) {
+                const int k = sp[s].gather == PIC_GATHER_MOMENTUM && (c->guard == 2) == (sp[s].shape == 3) ? sp[s].shape : 0;
+                c->push_only = c->push_only < 0 || c->push_only == k ? k : 0;
+            }
+        c->push_only = std::max(c->push_only, 0);
         if ((1 << c->log2S) != c->S || !push_supported(c->LX, c->LY, c->LZ, c->threads, c->guard))
             return bail(PIC_ERR_ARG);
         if (push_smem_bytes(c->LX, c->LY, c->LZ, c->threads, c->guard) > c->smem_optin)

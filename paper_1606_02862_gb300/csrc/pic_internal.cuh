@@ -89,6 +89,8 @@ struct StepDev {
     int LX, LY, LZ, S, log2S;  // supercell edges, frame size
     int guard;                 // field guard cells below the interior (1, or 2 with PCS)
     int nboxes, nsc, nspecies, nlists;
+    int push_only;             // 1, 2, 3: every mobile species has that shape (CIC, TSC, PCS) and the
+                               // momentum-conserving gather; 0: a mix
     float dt;
     float move[3];            // dt / h_d
     const BoxDev* boxes;      // [nboxes]
@@ -225,7 +227,8 @@ cudaError_t configure_yee_fused();
 // the whole field update of one step from p.src into f.dst: antenna (into J),
 // k_yee_fused, absorber (on dst); p supplies dt, 1/h, the antenna and absorber
 cudaError_t launch_yee_fused(const YeePlan& p, const FusedPlan& f, cudaStream_t st);
-cudaError_t configure_push(int LX, int LY, int LZ, int threads, int guard, int* per_sm);
+// only: see StepDev::push_only
+cudaError_t configure_push(int LX, int LY, int LZ, int threads, int guard, int only, int* per_sm);
 // the E/B tile the push stages per supercell: row pitch px (floats), ty rows, tz planes
 void push_tile_box(int LX, int LY, int LZ, int guard, int* px, int* ty, int* tz);
 cudaError_t launch_push_deposit(const StepDev& d, int threads, int grid, cudaStream_t st);
