@@ -196,34 +196,42 @@ __global__ void __launch_bounds__(256) k_yee_b(const YeeArgs a)
 // step's current, t = (n + 1/2) dt, n = steps taken before it (step_no was
 // advanced earlier in the step).  Runs before the E update, which folds it
 // in with the deposits.  FP64 throughout: omega t reaches thousands of
-// radians.  One thread per (box, x, z), grid-stride.
-__device__ __forceinline__ float antenna_current(const YeeArgs& a, const BoxDev& b, int x, int z)
-{
-    const OpenYDev& o = b.oy;
-    const double t = ((double)(*a.step_no) - 0.5) * a.dt_d;
-    const double T = o.ant_tau > 0.0 ? exp(-((t - o.ant_t0) / o.ant_tau) * ((t - o.ant_t0) / o.ant_tau)) : 1.0;
-    double G = 1.0;
-    if (o.ant_w0 > 0.0) {
-        const double px = ((double)x + 0.5) * a.dx_d[0] - o.ant_xc;
-        const double pz = (double)z * a.dx_d[2] - o.ant_zc;
-        G = exp(-(px * px + pz * pz) / (o.ant_w0 * o.ant_w0));
-    }
-    return (float)(o.ant_J0 * G * T * cos(o.ant_omega * (t - o.ant_t0)));
-}
+// radians.  One thread per (box, x, z), grid-stride.  The FP64 pipe bounds it,
+// so the two factors of the time alone are formed once per block (by two of
+// its warps) and the points are spread over every SM.
+constexpr int kAntThreads = 128, kAntBlocks = 304;
 
-__global__ void __launch_bounds__(256) k_antenna(const YeeArgs a)
+__global__ void __launch_bounds__(kAntThreads) k_antenna(const YeeArgs a)
 {
+    __shared__ double time_factor[2];
     for (int box = 0; box < a.nboxes; ++box) {
         const BoxDev& b = a.boxes[box];
-        const int j = b.oy.ant_j;
-        if (j < 0)
-            continue;
+        const OpenYDev o = b.oy;
+        const int j = o.ant_j;
         const int64_t n = (int64_t)b.nx * b.nz;
-        for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-             t += (int64_t)gridDim.x * blockDim.x) {
-            const int x = (int)(t % b.nx), z = (int)(t / b.nx);
-            b.J[padded_index(b, x, j, z)] += antenna_current(a, b, x, z);
+        const int64_t t0 = blockIdx.x * (int64_t)kAntThreads;
+        if (j < 0 || t0 >= n)
+            continue;
+        if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) {
+            const double t = ((double)(*a.step_no) - 0.5) * a.dt_d;
+            if (threadIdx.x == 0)
+                time_factor[0] = o.ant_tau > 0.0 ? exp(-((t - o.ant_t0) / o.ant_tau) * ((t - o.ant_t0) / o.ant_tau)) : 1.0;
+            else
+                time_factor[1] = cos(o.ant_omega * (t - o.ant_t0));
         }
+        __syncthreads();
+        const double T = time_factor[0], C = time_factor[1];
+        for (int64_t t = t0 + threadIdx.x; t < n; t += (int64_t)kAntBlocks * kAntThreads) {
+            const int x = (int)(t % b.nx), z = (int)(t / b.nx);
+            double G = 1.0;
+            if (o.ant_w0 > 0.0) {
+                const double px = ((double)x + 0.5) * a.dx_d[0] - o.ant_xc;
+                const double pz = (double)z * a.dx_d[2] - o.ant_zc;
+                G = exp(-(px * px + pz * pz) / (o.ant_w0 * o.ant_w0));
+            }
+            b.J[padded_index(b, x, j, z)] += (float)(o.ant_J0 * G * T * C);
+        }
+        __syncthreads();  // time_factor is free for the next box
     }
 }
 
@@ -300,6 +308,22 @@ __global__ void __launch_bounds__(256, 4) k_yee_e(const YeeArgs a)
     }
 }
 
+// y absorber: every E and B value whose staggered y position lies in a
+// damping layer is multiplied by exp(-sigma d^2) (d = depth in the layer, 0
+// at its inner edge, 1 at the face), images included.  The fused field
+// update multiplies the values as it stores them (1 outside the layers); after
+// the in-place one k_absorb_y does.
+__device__ __forceinline__ float absorb_factor(float y, int ny, int A, float sigma)
+{
+    float depth = 0.0f;
+    if (y < (float)A)
+        depth = ((float)A - y) / (float)A;
+    else if (y > (float)(ny - A))
+        depth = (y - (float)(ny - A)) / (float)A;
+    depth = fminf(depth, 1.0f);
+    return expf(-sigma * depth * depth);
+}
+
 // ------------------------------------------------------------ fused field update
 //
 // The whole field half of the cycle in one kernel, from one buffer pair into
@@ -325,13 +349,18 @@ __global__ void __launch_bounds__(256, 4) k_yee_e(const YeeArgs a)
 // an iteration ahead: the blocks at the faces set the pace of the others).
 // HBM traffic per cell: E^n, B^n, J read and E^{n+1}, B^{n+1} written, 60 bytes
 // (the three in-place kernels move 120); the rim comes from L2.  The arithmetic
-// of every value is that of k_yee_b, k_yee_e, k_yee_b, to the last bit.
-// Measured: 256^3 0.243 ms (4.1 TB/s of the 60 bytes; in place 0.450), 192x768x192
-// 0.404 ms (0.739), 128^3 0.059 ms (0.064).  With every stage's values of its own
+// of every value is that of k_yee_b, k_yee_e, k_yee_b, to the last bit.  A block
+// whose rows reach into a y absorber's layer multiplies what it stores by the
+// column's two factors (a pass over the layers less: with the antenna's factors
+// of time once per block, the field update of a 64x512x64 box with both 0.091 ->
+// 0.077 ms).
+// Measured: 256^3 0.240 ms (4.2 TB/s of the 60 bytes; in place 0.450), 192x768x192
+// 0.401 ms (0.739), 128^3 0.057 ms (0.064).  With every stage's values of its own
 // column in shared memory too (39 shared loads per cell instead of 20), 24
 // planes per chunk and the image code in every block it took 0.400 ms, 0.698
 // ms and 0.067 ms.  What bounds it now is the blocks at the box faces and the
-// barrier of every iteration; tiles of 6, 12, 14 and 16 rows were no faster.
+// barrier of every iteration; tiles of 6, 12, 14 and 16 rows were no faster, and
+// the absorber's factors in the march of every block cost 2 %.
 constexpr int kFX = kFusedTX, kFY = kFusedTY;
 constexpr int kHX = kFX + 2, kHY = kFY + 2, kHN = kHX * kHY;  // columns x0-1 .. x0+kFX, y0-1 .. y0+kFY
 constexpr int kFWarps = kHY + (2 * kHY + 31) / 32;            // a warp per row, then the rim columns
@@ -377,7 +406,7 @@ int fused_resident() { return kFBlocksSM; }
 // J gathers guard images and E, B are stored to them as well; without it (most
 // blocks of a large box) none of that code is in the loop.  Returns false when
 // a wait gave up.
-template <int G, bool FACES>
+template <int G, bool FACES, bool ABSORB>
 __device__ __forceinline__ bool fused_march(const FusedArgs& a, FusedSmem& sm, int box, int x0, int y0, int zc0, int zc1)
 {
     // the box's geometry and arrays in registers (stores through the field
@@ -412,6 +441,12 @@ __device__ __forceinline__ bool fused_march(const FusedArgs& a, FusedSmem& sm, i
     const bool edge = dx != 0 || dy != 0 || x >= nx || y >= ny;
     auto inner_plane = [&](int z) { return z >= hyz && z < nz - G; };
     const int64_t ccol = (int64_t)(yc + G) * px + (xc + G);
+    // the absorber's factors of this column (1: none): integer and half y positions
+    float fi = 1.0f, fh = 1.0f;
+    if (ABSORB && dob) {
+        fi = absorb_factor((float)y, ny, bt.oy.abs_cells, bt.oy.abs_sigma);
+        fh = absorb_factor((float)y + 0.5f, ny, bt.oy.abs_cells, bt.oy.abs_sigma);
+    }
     auto put = [&](float* p, float v0, float v1, float v2) {
         p[0] = v0;
         p[pc] = v1;
@@ -561,14 +596,17 @@ __device__ __forceinline__ bool fused_march(const FusedArgs& a, FusedSmem& sm, i
             }
             if (dob) {
                 if (s < zc1)
-                    store3(pe, s, nex, ney, nez);
+                    store3(pe, s, ABSORB ? nex * fi : nex, ABSORB ? ney * fh : ney, ABSORB ? nez * fi : nez);
                 // B^{n+1}(s-1) = B^{n+1/2} - tau curl E^{n+1}
                 if (s > zc0) {
                     const float* X0 = sm.e1[(s - 1) & 1][0] + h;
                     const float cx = (X0[2 * kHN + kHX] - fz) * ih1 - (ney - fy) * ih2;
                     const float cy = (nex - fx) * ih2 - (X0[2 * kHN + 1] - fz) * ih0;
                     const float cz = (X0[kHN + 1] - fy) * ih0 - (X0[kHX] - fx) * ih1;
-                    store3(pb, s - 1, qx - tau * cx, qy - tau * cy, qz - tau * cz);
+                    {
+                        const float vx = qx - tau * cx, vy = qy - tau * cy, vz = qz - tau * cz;
+                        store3(pb, s - 1, ABSORB ? vx * fh : vx, ABSORB ? vy * fi : vy, ABSORB ? vz * fh : vz);
+                    }
                 }
             }
         }
@@ -612,8 +650,12 @@ __global__ void __launch_bounds__(kFT, kFBlocksSM) k_yee_fused(const FusedArgs a
     // the E update: none of them within the reach of a face's guards
     const bool faces = x0 < GuardsOf<G>::hx || x0 + kFX >= b.nx - G || y0 < GuardsOf<G>::hyz ||
                        y0 + kFY >= b.ny - G || zc0 < GuardsOf<G>::hyz || zc1 >= b.nz - G;
-    const bool ok = faces ? fused_march<G, true>(a, sm, box, x0, y0, zc0, zc1)
-                          : fused_march<G, false>(a, sm, box, x0, y0, zc0, zc1);
+    // rows y0 .. y0 + kFY - 1 reach into an absorber layer
+    const int A = b.oy.abs_cells;
+    const bool absorb = A > 0 && (y0 < A || y0 + kFY > b.ny - A);
+    const bool ok = absorb ? fused_march<G, true, true>(a, sm, box, x0, y0, zc0, zc1)
+                           : (faces ? fused_march<G, true, false>(a, sm, box, x0, y0, zc0, zc1)
+                                    : fused_march<G, false, false>(a, sm, box, x0, y0, zc0, zc1));
     if (!ok && threadIdx.x == 0)
         atomicOr(a.status, ST_TIMEOUT);
 }
@@ -630,55 +672,41 @@ cudaError_t configure_yee_fused()
     return e;
 }
 
-// y absorber: every E and B value whose staggered y position lies in a
-// damping layer is multiplied by exp(-sigma d^2) (d = depth in the layer, 0
-// at its inner edge, 1 at the face), images included.  Work: the 2A planes
-// j < A and j >= ny - A of each box with a layer, 256 cells per block.
-__device__ __forceinline__ float absorb_factor(float y, int ny, int A, float sigma)
-{
-    float depth = 0.0f;
-    if (y < (float)A)
-        depth = ((float)A - y) / (float)A;
-    else if (y > (float)(ny - A))
-        depth = (y - (float)(ny - A)) / (float)A;
-    depth = fminf(depth, 1.0f);
-    return expf(-sigma * depth * depth);
-}
-
+// The in-place update's absorber: a block per 32 x 8 cells (x, layer row) of
+// the 2A rows j < A and j >= ny - A of a plane of each box with a layer.
 int absorber_blocks(const BoxDev& b)
 {
-    const int A = b.oy.abs_cells;
-    if (A <= 0)
-        return 0;
-    const int64_t cells = (int64_t)2 * A * b.nx * b.nz;
-    return (int)((cells + 255) / 256);
+    return ((b.nx + 31) / 32) * ((2 * b.oy.abs_cells + 7) / 8) * b.nz;
 }
 
 __global__ void __launch_bounds__(256) k_absorb_y(const BoxDev* boxes, const int* off, int nboxes)
 {
     const int box = find_box(off, nboxes, blockIdx.x);
     const BoxDev& b = boxes[box];
-    const int A = b.oy.abs_cells;
-    const int64_t t = (int64_t)(blockIdx.x - off[box]) * 256 + threadIdx.x;
-    if (A <= 0 || t >= (int64_t)2 * A * b.nx * b.nz)
-        return;
+    const int A = b.oy.abs_cells, local = blockIdx.x - off[box];
+    const int nbx = (b.nx + 31) / 32, nbp = (2 * A + 7) / 8;
     CellAt c;
-    c.x = (int)(t % b.nx);
-    const int p = (int)((t / b.nx) % (2 * A));
-    c.z = (int)(t / ((int64_t)b.nx * 2 * A));
+    c.x = (local % nbx) * 32 + threadIdx.x;
+    const int p = (local / nbx) % nbp * 8 + threadIdx.y;
+    c.z = local / (nbx * nbp);
     c.y = p < A ? p : b.ny - 2 * A + p;
-    c.ok = true;
+    c.ok = c.x < b.nx && p < 2 * A;
+    if (!c.ok)
+        return;
     const int64_t pc = padded_cells(b);
     const int64_t i = padded_index(b, c.x, c.y, c.z);
+    float* __restrict__ E = b.E;
+    float* __restrict__ B = b.B;
+    const float ex = E[i], ey = E[pc + i], ez = E[2 * pc + i], bx = B[i], by = B[pc + i], bz = B[2 * pc + i];
     const float s = b.oy.abs_sigma;
     const float fi = absorb_factor((float)c.y, b.ny, A, s);          // Ex, Ez, By
     const float fh = absorb_factor((float)c.y + 0.5f, b.ny, A, s);   // Ey, Bx, Bz
-    store_with_images(b, b.E, c, b.E[i] * fi);
-    store_with_images(b, b.E + pc, c, b.E[pc + i] * fh);
-    store_with_images(b, b.E + 2 * pc, c, b.E[2 * pc + i] * fi);
-    store_with_images(b, b.B, c, b.B[i] * fh);
-    store_with_images(b, b.B + pc, c, b.B[pc + i] * fi);
-    store_with_images(b, b.B + 2 * pc, c, b.B[2 * pc + i] * fh);
+    store_with_images(b, E, c, ex * fi);
+    store_with_images(b, E + pc, c, ey * fh);
+    store_with_images(b, E + 2 * pc, c, ez * fi);
+    store_with_images(b, B, c, bx * fh);
+    store_with_images(b, B + pc, c, by * fi);
+    store_with_images(b, B + 2 * pc, c, bz * fh);
 }
 
 cudaError_t launch_yee_mixed_part(const YeePlan& p, int part, cudaStream_t st)
@@ -693,13 +721,13 @@ cudaError_t launch_yee_mixed_part(const YeePlan& p, int part, cudaStream_t st)
         yb<<<p.nblocks, blk, 0, st>>>(a);
     } else if (part == 1) {
         if (p.antenna)
-            k_antenna<<<64, 256, 0, st>>>(a);
+            k_antenna<<<kAntBlocks, kAntThreads, 0, st>>>(a);
         a.tau = p.dt;
         ye<<<p.nblocks, blk, 0, st>>>(a);
     } else {
         yb<<<p.nblocks, blk, 0, st>>>(a);
         if (p.abs_nblocks > 0)
-            k_absorb_y<<<p.abs_nblocks, 256, 0, st>>>(p.boxes, p.abs_off, p.nboxes);
+            k_absorb_y<<<p.abs_nblocks, blk, 0, st>>>(p.boxes, p.abs_off, p.nboxes);
     }
     return cudaGetLastError();
 }
@@ -719,7 +747,7 @@ cudaError_t launch_yee_fused(const YeePlan& p, const FusedPlan& f, cudaStream_t 
     if (p.antenna) {
         YeeArgs ya{f.src, p.blk_off, p.nboxes, p.dt, {p.ih[0], p.ih[1], p.ih[2]},
                    p.step_no, p.dt_d, {p.dx_d[0], p.dx_d[1], p.dx_d[2]}};
-        k_antenna<<<64, 256, 0, st>>>(ya);
+        k_antenna<<<kAntBlocks, kAntThreads, 0, st>>>(ya);
     }
     FusedArgs a{f.src, f.dst, f.maps, f.blk_off, p.nboxes, f.tz, p.dt, 0.5f * p.dt, {p.ih[0], p.ih[1], p.ih[2]},
                 f.status};
@@ -727,8 +755,6 @@ cudaError_t launch_yee_fused(const YeePlan& p, const FusedPlan& f, cudaStream_t 
         k_yee_fused<2><<<f.nblocks, kFT, sizeof(FusedSmem), st>>>(a);
     else
         k_yee_fused<1><<<f.nblocks, kFT, sizeof(FusedSmem), st>>>(a);
-    if (p.abs_nblocks > 0)
-        k_absorb_y<<<p.abs_nblocks, 256, 0, st>>>(f.dst, p.abs_off, p.nboxes);
     return cudaGetLastError();
 }
 

@@ -2226,9 +2226,9 @@ pic_status pic_info(pic_ctx* c, int32_t key, int64_t* out)
             // push; frame maintenance; Yee x3; antenna; y absorber;
             // a subdomain slab adds its 16 halo pack/unpack launches (J, B, E, B:
             // two faces each way) and 2 migrant accepts
-            // (the fused field update: one kernel for the three)
+            // (the fused field update: one kernel for the three and the absorber)
             const bool fused = c->fused_ready;
-            *out = 1 + frame_launches(c->nlists) + (fused ? 1 : 3) + (c->any_antenna ? 1 : 0) + (c->abs_nblocks > 0 ? 1 : 0) +
+            *out = 1 + frame_launches(c->nlists) + (fused ? 1 : 3) + (c->any_antenna ? 1 : 0) + (!fused && c->abs_nblocks > 0 ? 1 : 0) +
                    (c->sub_z ? 18 : 0);
         } else {
             int64_t k = 0;

@@ -225,7 +225,7 @@ int fused_resident();
 size_t fused_smem_bytes();
 cudaError_t configure_yee_fused();
 // the whole field update of one step from p.src into f.dst: antenna (into J),
-// k_yee_fused, absorber (on dst); p supplies dt, 1/h, the antenna and absorber
+// k_yee_fused with the absorber; p supplies dt, 1/h and the antenna
 cudaError_t launch_yee_fused(const YeePlan& p, const FusedPlan& f, cudaStream_t st);
 // only: see StepDev::push_only
 cudaError_t configure_push(int LX, int LY, int LZ, int threads, int guard, int only, int* per_sm);

@@ -255,3 +255,31 @@ def test_fused_tiles_and_faces(n, shape):
         finally:
             ctx.close()
     print("fused tiles errors:", n, _agree(states[0], states[1], wl))
+
+
+def test_absorber_layers_of_the_fused_update():
+    """Layers that end inside a tile, fill half a box or are absent, in one
+    context without particles: the same E, B and J (the antenna's) as the
+    in-place kernels, whose absorber is a pass of its own, to the last bit."""
+    require_gpu()
+    from paper_1606_02862_gb300 import pic
+    from paper_1606_02862_gb300 import workloads as W
+
+    rng = np.random.default_rng(9)
+    none = (np.empty((0, 3)), np.empty((0, 3)), np.empty(0))
+    boxes = [W.BoxInit(*n, particles=[none], E=rng.normal(0, 1, (3, n[2], n[1], n[0])))
+             for n in ((40, 28, 12), (32, 20, 8), (16, 24, 8), (68, 48, 40))]
+    wl = W.Workload("absorbers", W.DT_HALF_COURANT, [W.SpeciesDef("e", -1.0, 1.0, 2)], boxes)
+    states = []
+    for form in (pic.FIELD_UPDATE_FUSED, pic.FIELD_UPDATE_IN_PLACE):
+        ctx = ctx_from(wl, field_update=form)
+        try:
+            for b, cells in enumerate((5, 0, 12, 13)):
+                ctx.set_boundary(b, open_y=True, absorber_cells=cells, absorber_sigma=1.3)
+                ctx.set_antenna(b, plane_y=9, E0=0.7, omega=0.4, w0=6.0, xc=8.0, zc=4.0, tau=20.0, t0=3.0)
+            ctx.step(4)
+            states.append([ctx.read_fields(b, k) for b in range(len(boxes)) for k in range(3)])
+        finally:
+            ctx.close()
+    for f, i in zip(*states):
+        assert np.array_equal(f, i)
