@@ -62,6 +62,7 @@ struct pic_ctx {
     // allocations
     std::vector<void*> allocs;
     unsigned* status_d = nullptr;
+    unsigned* status_h = nullptr;  // page-locked copy, read at every synchronisation
     double* diag_d = nullptr;
     double* rho_d = nullptr;
     int* ioff_d = nullptr;  // scratch ints for read-back offsets
@@ -131,6 +132,7 @@ struct pic_ctx {
     cudaGraph_t graph[2] = {nullptr, nullptr};
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     cudaGraphNode_t evnode[2][4] = {};
+    bool ev_set[2] = {false, false};  // the graph's event nodes point at a step's own events
     cudaEvent_t placeholder[8] = {};
     bool graph_failed = false;
     // fused field update (pic_options.field_update 0): a second field buffer
@@ -150,6 +152,7 @@ struct pic_ctx {
     cudaGraph_t pgraph[2] = {nullptr, nullptr};
     cudaGraphExec_t pgexec[2] = {nullptr, nullptr};
     cudaGraphNode_t pevnode[2][8] = {};
+    bool pev_set[2] = {false, false};
     // plain form
     std::vector<PlainBox> pboxes;
     // stage timing
@@ -263,6 +266,7 @@ void destroy_graphs(pic_ctx* c)
             cudaGraphDestroy(c->pgraph[p]);
         c->pgexec[p] = nullptr;
         c->pgraph[p] = nullptr;
+        c->ev_set[p] = c->pev_set[p] = false;  // captured with the placeholders
     }
 }
 
@@ -341,9 +345,10 @@ pic_status ensure_ioff(pic_ctx* c, int64_t n)
 
 pic_status status_check(pic_ctx* c)
 {
+    // the copy is part of the stream's work, so that one wait covers both
+    CK(cudaMemcpyAsync(c->status_h, c->status_d, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    unsigned st = 0;
-    CK(cudaMemcpy(&st, c->status_d, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    const unsigned st = *c->status_h;
     if (st == 0)
         return PIC_OK;
     if (st & ST_FRAME_POOL)
@@ -791,16 +796,20 @@ pic_status capture_pair_graphs(pic_ctx* c)
 
 pic_status launch_pair_graph(pic_ctx* c, int p, cudaEvent_t* ev)
 {
-    for (int k = 0; k < 8; ++k)
-        CK(cudaGraphExecEventRecordNodeSetEvent(c->pgexec[p], c->pevnode[p][k], ev ? ev[k] : c->placeholder[k]));
+    if (ev || c->pev_set[p])
+        for (int k = 0; k < 8; ++k)
+            CK(cudaGraphExecEventRecordNodeSetEvent(c->pgexec[p], c->pevnode[p][k], ev ? ev[k] : c->placeholder[k]));
+    c->pev_set[p] = ev != nullptr;
     CK(cudaGraphLaunch(c->pgexec[p], c->stream));
     return PIC_OK;
 }
 
 pic_status launch_graph(pic_ctx* c, int p, cudaEvent_t* ev)
 {
-    for (int k = 0; k < 4; ++k)
-        CK(cudaGraphExecEventRecordNodeSetEvent(c->gexec[p], c->evnode[p][k], ev ? ev[k] : c->placeholder[k]));
+    if (ev || c->ev_set[p])
+        for (int k = 0; k < 4; ++k)
+            CK(cudaGraphExecEventRecordNodeSetEvent(c->gexec[p], c->evnode[p][k], ev ? ev[k] : c->placeholder[k]));
+    c->ev_set[p] = ev != nullptr;
     CK(cudaGraphLaunch(c->gexec[p], c->stream));
     return PIC_OK;
 }
@@ -1241,6 +1250,11 @@ pic_status pic_create(const pic_grid* grids, int32_t nboxes, const double dx[3],
             return bail(PIC_ERR_CUDA);
         }
         c->own_stream = true;
+    }
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->status_h), sizeof(unsigned), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        c->status_h = nullptr;
+        return bail(PIC_ERR_CUDA);
     }
     if (dalloc(c, &c->status_d, 1) != PIC_OK || dalloc(c, &c->diag_d, 4) != PIC_OK)
         return bail(PIC_ERR_OOM);
@@ -2482,6 +2496,8 @@ void pic_destroy(pic_ctx* c)
     std::vector<void*> all = c->allocs;
     for (void* p : all)
         raw_free(c, p);
+    if (c->status_h)
+        cudaFreeHost(c->status_h);
     if (c->own_stream && c->stream)
         cudaStreamDestroy(c->stream);
     cudaGetLastError();
