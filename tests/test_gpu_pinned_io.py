@@ -209,3 +209,30 @@ def test_pinned_field_read():
             assert np.array_equal(out.numpy(), ref)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("words", [1, 7, 15])
+def test_pinned_read_at_any_word(words):
+    """Destinations that start `words` words into a 128-byte line, each array
+    at another offset: the same values as into line-aligned arrays, and nothing
+    written before or behind them (supercell runs of odd lengths)."""
+    torch = require_gpu()
+    n, x, u, w = _state(seed=11, ppc=3)
+    keep = np.random.default_rng(2).random(x.shape[0]) < 0.6
+    x, u, w = x[keep], u[keep], w[keep]
+    m = x.shape[0]
+    ctx = _ctx(n)
+    try:
+        ctx.load_particles(0, 0, x, u, w)
+        ctx.step(2)
+        ref = _read(torch, ctx, m, True)
+        sizes, types = (3 * m, 3 * m, m, m), (torch.float64,) * 3 + (torch.int64,)
+        offs = [(words + 3 * k) % 16 for k in range(4)]
+        bufs = [torch.full((s + 32,), -77, dtype=t, pin_memory=True) for s, t in zip(sizes, types)]
+        assert ctx.read_particles_ptr(0, 0, m, *(b.data_ptr() + 8 * o for b, o in zip(bufs, offs))) == m
+        for b, o, s, r in zip(bufs, offs, sizes, ref):
+            got = b.numpy()
+            assert np.array_equal(got[o:o + s], np.asarray(r).reshape(-1))
+            assert np.all(got[:o] == -77) and np.all(got[o + s:] == -77)
+    finally:
+        ctx.close()
