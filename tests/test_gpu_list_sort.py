@@ -40,3 +40,34 @@ def test_sorted_lists(orc, n, shape, sc, threads):
         compare_box(st, ids, ctx, wl, 0, tol_field=1e-5, tol_x=1e-5, tol_u=1e-5)
     finally:
         ctx.close()
+
+
+def test_resting_lists_are_left_alone(orc):
+    """A species at rest beside a fast one, a sort due on every step: the lists
+    that nothing joins keep their order, the others are sorted, and both match
+    the FP64 oracle over the next step."""
+    require_gpu()
+    from paper_1606_02862_gb300 import workloads as W
+
+    rng = np.random.default_rng(8)
+    N = 16
+    xs = [rng.random((900, 3)) * N for _ in range(2)]
+    us = [rng.normal(0, 0.5, (900, 3)), np.zeros((900, 3))]
+    box = W.BoxInit(N, N, N, particles=[(x, u, np.full(900, 0.01)) for x, u in zip(xs, us)])
+    sp = [W.SpeciesDef("e", -1.0, 1.0, 2), W.SpeciesDef("i", 1.0, 1e9, 2)]
+    wl = W.Workload("rest_test", W.DT_HALF_COURANT, sp, [box])
+    ctx = ctx_from(wl, sc=(8, 4, 4), threads_per_sc=256, sort_every=1)
+    try:
+        ctx.step(1)
+        before = [ctx.read_particles(0, s, ids=True)["id"] for s in range(2)]
+        ctx.step(3)
+        after = [ctx.read_particles(0, s, ids=True)["id"] for s in range(2)]
+        assert np.array_equal(before[1], after[1])
+        assert not np.array_equal(before[0], after[0])
+        assert np.array_equal(np.sort(after[0]), np.sort(before[0]))
+        st, ids = oracle_state_from_gpu(orc, ctx, wl, 0)
+        ctx.step(1)
+        st.step(1)
+        compare_box(st, ids, ctx, wl, 0, tol_field=1e-5, tol_x=1e-5, tol_u=1e-5)
+    finally:
+        ctx.close()
