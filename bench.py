@@ -947,7 +947,7 @@ def main():
                     help="skip the short runs of the other configurations in the default line")
     ap.add_argument("--leg-steps", type=int, default=20)
     ap.add_argument("--sort-every", type=int, default=0,
-                    help="steps between sort passes of the push (0: the library's default, 4)")
+                    help="steps between sorts of the frame lists (0: the library's default, 4)")
     ap.add_argument("--diag-every", type=int, default=0,
                     help="--workload runs: FP64 diagnostics every this many steps")
     ap.add_argument("--shape", default="tsc", choices=["tsc", "cic", "pcs"],

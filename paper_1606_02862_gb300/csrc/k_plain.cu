@@ -191,7 +191,7 @@ __device__ __forceinline__ void deposit64(double* J, double cf, const int64_t* n
 // the transverse factors in the two-term form (deposit64), and the current on 3
 // (TSC) or 2 (CIC) nodes per axis, with a fourth (third) only for the axes where
 // the move leaves the old support's window.  2.1 million TSC particles in 64^3
-// cells: 8.61 -> 2.4 ms per step, 0.88 G particles/s.
+// cells: 8.61 -> 2.45 ms per step, 0.86 G particles/s.
 template <int SHAPE>
 __global__ void __launch_bounds__(128, 3) k_plain_push(const PlainPushArgs a)
 {
