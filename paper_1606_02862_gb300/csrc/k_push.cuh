@@ -388,13 +388,16 @@ __device__ __forceinline__ float rsqrt_ge1(float x)
 }
 
 // 2 / x for x >= 1: the approximate reciprocal and one step of Newton's
-// iteration for it
+// iteration for it, of x / 4, whose reciprocal is in FP32's normal range for
+// every finite x.  An x that overflowed gives 0, as the division does (Newton's
+// step alone would give 0 * infinity).
 __device__ __forceinline__ float two_over_ge1(float x)
 {
+    const float h = 0.25f * x;
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    r = fmaf(r, fmaf(-x, r, 1.0f), r);
-    return r + r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
+    r = fmaf(r, fmaf(-h, r, 1.0f), r);
+    return x == INFINITY ? 0.0f : 0.5f * r;
 }
 
 // Esirkepov's transverse factor S0e S0f + (DSe S0f + S0e DSf)/2 + DSe DSf / 3
