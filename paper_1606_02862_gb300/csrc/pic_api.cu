@@ -73,6 +73,7 @@ struct pic_ctx {
     int LX = 4, LY = 4, LZ = 4, S = 64, log2S = 6, threads = 64;
     int guard = 1;  // field guard cells below the interior: 2 when a species has the PCS shape
     int push_grid = 0;
+    int place_grid = 0;  // of place_blocks, as the step graphs were captured with it
     int push_only = 0;  // StepDev::push_only
     std::vector<BoxDev> boxes_h;
     BoxDev* boxes_d = nullptr;
@@ -613,7 +614,8 @@ pic_status enqueue_stage(pic_ctx* c, int stage, int parity, int fsrc = -1)
         CK(launch_push_deposit(d, c->threads, c->push_grid, c->stream));
         return PIC_OK;
     case PIC_STAGE_FRAMES:
-        CK(launch_frames(d, place_blocks(c), sort_blocks(c), c->stream));
+        // (a subdomain slab's particles come and go uncounted)
+        CK(launch_frames(d, c->sub_z ? 4 * c->nsm : c->place_grid, sort_blocks(c), c->stream));
         return PIC_OK;
     default:
         CK(launch_yee_mixed_part(yee_plan(c), stage - PIC_STAGE_B_FIRST, c->stream));
@@ -672,6 +674,15 @@ pic_status prepare_mixed(pic_ctx* c)
     int per_sm = 0;
     CK(configure_push(c->LX, c->LY, c->LZ, c->threads, c->guard, c->push_only, &per_sm));
     c->push_grid = std::max(1, per_sm) * c->nsm;
+    // The step graphs hold the placing kernel's grid of their capture: a load
+    // that more than doubles it drops them (doublings, so that a load in many
+    // pieces costs a few captures in all).  64^3, 64 particles and then 6.3
+    // million into preset buffers: 0.08 ms of frame maintenance a step, 0.95
+    // with the grid of the first load.
+    if (place_blocks(c) > 2 * c->place_grid) {
+        destroy_graphs(c);
+        c->place_grid = place_blocks(c);
+    }
     // freshly loaded particles sit unsorted at the ends of their lists
     CK(configure_sort());
     CK(launch_sort(make_step(c, c->parity), 4 * c->nsm, c->stream));
