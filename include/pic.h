@@ -141,10 +141,11 @@ typedef struct {
     int32_t track_ids;      /* nonzero: carry a particle id (load order) through the frames */
     int32_t use_graph;      /* nonzero: pic_step replays a captured CUDA graph of one step */
     int32_t sort_every;     /* mixed form: every this many steps the frame lists are counting-sorted by
-                               nearest node (TSC) / cell (CIC, PCS), whole lists after the step's frame
-                               maintenance (TSC, PCS) or 256 particles at a time in the push (CIC); the
-                               steps between push the lists in stored order; 0 = 4, 1 = sort on every
-                               step (results agree up to FP32 summation order) */
+                               nearest node (TSC) / cell (CIC, PCS): after the step's frame maintenance
+                               the whole lists that particles joined since their last sort (TSC, PCS),
+                               or every list, 256 particles at a time, in the push (CIC); the steps
+                               between push the lists in stored order; 0 = 4, 1 = sort on every step
+                               (results agree up to FP32 summation order) */
     int32_t field_update;   /* mixed form, the field half of the step (Sec. 4, Yee solver), one of
                                PIC_FIELD_UPDATE_* (above); 0 = chosen at the first step */
     int32_t reserved;       /* 0 */

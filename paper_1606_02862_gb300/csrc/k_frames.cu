@@ -177,10 +177,12 @@ __device__ __forceinline__ void apply_lists(const StepDev& d, int4 tot, int base
             d.released[off.z + (k - nf_new)] = src[k];
         d.foff_next[L] = off.x;
         d.nframes[L] = nf_new;
-        const int c = d.count[L];
+        const int c = d.count[L], arrivals = d.narrive[L];
         d.abase[L] = c;
-        d.count[L] = c + d.narrive[L];
+        d.count[L] = c + arrivals;
         d.narrive[L] = 0;
+        if (arrivals > 0)
+            d.joined[L] = 1;
         off = off + need[i];
     }
 }
@@ -411,26 +413,26 @@ __device__ __forceinline__ void sort_run(const StepDev& d, SortSmem& sm, const i
     __syncthreads();  // the next run fills the stage and clears the histogram
 }
 
-// all: also the lists that no particle joined in this step.  A list's counts
-// are loaded while the block sorts the list before it.
+// The lists that particles joined since they were last sorted (all: every
+// list).  A list's counts are loaded while the block sorts the list before it.
 __device__ __forceinline__ void sort_lists(const StepDev& d, SortSmem& sm, const int* foff, const int* ftab, int first,
                                            int stride, bool all)
 {
     const int nitems = *d.nitems;
     const int total = nitems * d.nspecies;
     struct List {
-        int shape, n, off;  // n: 0 for a list that stays as it is
+        int L, shape, n, off;  // n: 0 for a list that stays as it is
     };
     auto fetch = [&](int t) {
-        List l{0, 0, 0};
+        List l{0, 0, 0, 0};
         if (t < total) {
             const int s = t / nitems;
-            const int L = s * d.nsc + d.items[t - s * nitems];
+            l.L = s * d.nsc + d.items[t - s * nitems];
             l.shape = d.sp[s].shape;
             if (d.sp[s].mobile && l.shape != 1) {
-                const int n = d.count[L], before = all ? -1 : d.abase[L];
-                l.off = foff[L];
-                l.n = n > 1 && n != before ? n : 0;
+                const int n = d.count[l.L];
+                l.off = foff[l.L];
+                l.n = n > 1 && (all || d.joined[l.L]) ? n : 0;
             }
         }
         return l;
@@ -445,6 +447,8 @@ __device__ __forceinline__ void sort_lists(const StepDev& d, SortSmem& sm, const
         const int per = ((l.n + runs - 1) / runs + 31) & ~31;
         for (int base = 0; base < l.n; base += per)
             sort_run(d, sm, ftab + l.off, base, min(per, l.n - base), l.shape);
+        if (threadIdx.x == 0)
+            d.joined[l.L] = 0;  // every thread read it before the barriers of sort_run
     }
 }
 
@@ -458,11 +462,13 @@ __global__ void __launch_bounds__(kSortThreads) k_sort(const StepDev d)
 // Last kernel of the maintenance: block 0 settles the free stack and the move
 // buffer; on every sort_every-th step the others sort the lists (the frame
 // table written in this step is the current one from here on).  A list that no
-// particle joined in this step is left as it is: its particles hardly move, so
-// its order is still good, and the slower they are the more rarely it is sorted
-// (cold ions: a thermal list of 1024 electrons gains about ten a step).  Half
-// ions, 64x512x64: maintenance 0.098 -> 0.061 ms a step; 192x768x192 0.144 ->
-// 0.121; 256^3 of electrons alone 0.562 ms either way.
+// particle joined since its last sort is left as it is: what moves within its
+// supercell reaches a face about as often as it changes node, so while nothing
+// joins, the order is nearly that of the sort, and the slower the particles are
+// the more rarely their lists are sorted (cold ions: a thermal list of 1024
+// electrons gains about ten a step).  Against sorting every list, maintenance
+// per step: half ions, 64x512x64 cells 0.087 -> 0.061 ms, 192x768x192 0.142 ->
+// 0.128; 256^3 cells of electrons alone 0.559 -> 0.569 (the marks).
 __global__ void __launch_bounds__(kSortThreads) k_finish(const StepDev d)
 {
     extern __shared__ __align__(16) unsigned char sort_smem[];
@@ -512,15 +518,17 @@ __global__ void k_clear_rows(const StepDev d, const BoxDev b, int rows)
 }
 
 // Moving window, part 2: the list of row scy takes over the list (count,
-// frames, frame-table offset) of row scy + rows, cyclically; the rows that
-// were emptied in part 1 come round to the top.  old3 = copies of count,
-// nframes and foff (nlists each), taken before the kernel.
-__global__ void k_rotate_lists(const StepDev d, const BoxDev b, const int* old3, int* foff, int rows)
+// frames, frame-table offset, mark of its arrivals) of row scy + rows,
+// cyclically; the rows that were emptied in part 1 come round to the top.
+// old4 = copies of count, nframes, foff and joined (nlists each), taken before
+// the kernel.
+__global__ void k_rotate_lists(const StepDev d, const BoxDev b, const int* old4, int* foff, int rows)
 {
     const int nbox = b.nscx * b.nscy * b.nscz;
-    const int* count_old = old3;
-    const int* nframes_old = old3 + d.nlists;
-    const int* foff_old = old3 + 2 * d.nlists;
+    const int* count_old = old4;
+    const int* nframes_old = old4 + d.nlists;
+    const int* foff_old = old4 + 2 * d.nlists;
+    const int* joined_old = old4 + 3 * d.nlists;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < d.nspecies * nbox;
          t += gridDim.x * blockDim.x) {
         const int s = t / nbox, loc = t % nbox;
@@ -531,6 +539,7 @@ __global__ void k_rotate_lists(const StepDev d, const BoxDev b, const int* old3,
         d.count[L] = count_old[Ls];
         d.nframes[L] = nframes_old[Ls];
         foff[L] = foff_old[Ls];
+        d.joined[L] = joined_old[Ls];
     }
 }
 
@@ -540,10 +549,10 @@ cudaError_t launch_clear_rows(const StepDev& d, const BoxDev& hb, int rows, cuda
     return cudaGetLastError();
 }
 
-cudaError_t launch_rotate_lists(const StepDev& d, const BoxDev& hb, const int* old3, int* foff,
+cudaError_t launch_rotate_lists(const StepDev& d, const BoxDev& hb, const int* old4, int* foff,
                                 int rows, cudaStream_t st)
 {
-    k_rotate_lists<<<256, 256, 0, st>>>(d, hb, old3, foff, rows);
+    k_rotate_lists<<<256, 256, 0, st>>>(d, hb, old4, foff, rows);
     return cudaGetLastError();
 }
 

@@ -85,7 +85,8 @@ struct pic_ctx {
     float *E_all = nullptr, *B_all = nullptr, *J_all = nullptr;
     int64_t field_floats = 0;  // per field, all boxes (3 components each)
     int nsc = 0, nlists = 0;
-    int *count = nullptr, *nframes = nullptr, *narrive = nullptr, *abase = nullptr;
+    int *count = nullptr, *nframes = nullptr, *narrive = nullptr, *abase = nullptr,
+        *joined = nullptr;
     int* foff[2] = {nullptr, nullptr};
     int* ftab[2] = {nullptr, nullptr};
     int *cell = nullptr, *pid = nullptr;
@@ -110,7 +111,7 @@ struct pic_ctx {
     bool any_antenna = false;
     float* shift_scratch = nullptr;    // moving window: copy of one box's field
     int64_t shift_scratch_floats = 0;
-    int* rot_scratch = nullptr;        // moving window: copies of count, nframes, foff
+    int* rot_scratch = nullptr;        // moving window: copies of count, nframes, foff, joined
     int sort_every = kDefaultSortEvery;
     unsigned* wmax_bits = nullptr;     // [kMaxSpecies] device
     float wmax[kMaxSpecies] = {};      // host copy: largest |weight| per species
@@ -431,6 +432,7 @@ StepDev make_step(const pic_ctx* c, int parity, bool alt = false)
     d.ftab_next = c->ftab[parity ^ 1];
     d.narrive = c->narrive;
     d.abase = c->abase;
+    d.joined = c->joined;
     d.free_stack = c->free_stack;
     d.free_top = c->free_top;
     d.released = c->released;
@@ -1376,6 +1378,7 @@ pic_status pic_create(const pic_grid* grids, int32_t nboxes, const double dx[3],
             dalloc(c, &c->items_d, nsc + 1) != PIC_OK || dalloc(c, &c->yee_off_d, nboxes + 1, false) != PIC_OK ||
             dalloc(c, &c->count, c->nlists) != PIC_OK || dalloc(c, &c->nframes, c->nlists) != PIC_OK ||
             dalloc(c, &c->narrive, c->nlists) != PIC_OK || dalloc(c, &c->abase, c->nlists) != PIC_OK ||
+            dalloc(c, &c->joined, c->nlists) != PIC_OK ||
             dalloc(c, &c->foff[0], c->nlists) != PIC_OK || dalloc(c, &c->foff[1], c->nlists) != PIC_OK ||
             dalloc(c, &c->free_top, 1) != PIC_OK || dalloc(c, &c->mv_count, 1) != PIC_OK ||
             dalloc(c, &c->blk_sums, nblk) != PIC_OK || dalloc(c, &c->blk_offs, nblk) != PIC_OK ||
@@ -1508,11 +1511,13 @@ pic_status pic_shift_window(pic_ctx* c, int32_t box, int32_t cells)
     CKS(status_check(c));
     c->parity ^= 1;
     if (!c->rot_scratch)
-        CKS(dalloc(c, &c->rot_scratch, 3 * (int64_t)c->nlists, false));
+        CKS(dalloc(c, &c->rot_scratch, 4 * (int64_t)c->nlists, false));
     CK(cudaMemcpyAsync(c->rot_scratch, c->count, sizeof(int) * c->nlists, cudaMemcpyDeviceToDevice, c->stream));
     CK(cudaMemcpyAsync(c->rot_scratch + c->nlists, c->nframes, sizeof(int) * c->nlists,
                        cudaMemcpyDeviceToDevice, c->stream));
     CK(cudaMemcpyAsync(c->rot_scratch + 2 * c->nlists, c->foff[c->parity], sizeof(int) * c->nlists,
+                       cudaMemcpyDeviceToDevice, c->stream));
+    CK(cudaMemcpyAsync(c->rot_scratch + 3 * (int64_t)c->nlists, c->joined, sizeof(int) * c->nlists,
                        cudaMemcpyDeviceToDevice, c->stream));
     d = make_step(c, c->parity);
     CK(launch_rotate_lists(d, b, c->rot_scratch, c->foff[c->parity], rows, c->stream));

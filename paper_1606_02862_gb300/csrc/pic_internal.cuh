@@ -118,6 +118,7 @@ struct StepDev {
     int* ftab_next;
     int* narrive;             // [nlists] arrivals in this step
     int* abase;               // [nlists] first slot of this step's arrivals
+    int* joined;              // [nlists] nonzero: particles joined the list since its last sort
     // frame pool free stack
     int* free_stack;          // [pool_frames]
     int* free_top;            // device scalar
@@ -268,7 +269,7 @@ cudaError_t launch_shift_fields(const BoxDev& b, float* F, const float* scratch,
 cudaError_t launch_clear_rows(const StepDev& d, const BoxDev& hb, int rows, cudaStream_t st);
 // rebuild d.items from the particle counts (launch_frame_apply does it too)
 cudaError_t launch_list_items(const StepDev& d, int blocks, cudaStream_t st);
-cudaError_t launch_rotate_lists(const StepDev& d, const BoxDev& hb, const int* old3, int* foff,
+cudaError_t launch_rotate_lists(const StepDev& d, const BoxDev& hb, const int* old4, int* foff,
                                 int rows, cudaStream_t st);
 cudaError_t launch_fields_to_padded(const BoxDev& b, int which, const double* src,
                                     cudaStream_t st);

@@ -71,3 +71,51 @@ def test_resting_lists_are_left_alone(orc):
         compare_box(st, ids, ctx, wl, 0, tol_field=1e-5, tol_x=1e-5, tol_u=1e-5)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("shift", [False, True])
+@pytest.mark.parametrize("shape", [2, 3])
+def test_arrivals_between_sorts(shape, shift):
+    """Particles at rest, and a few that enter the next supercell along y in the
+    second step and stay there; a sort is due on the fourth step, in which none
+    arrives.  It takes up the lists that they joined (a window shift in between
+    moves the lists by a row): every list is in order of its nodes (PCS: cells).
+    On the eighth step no list has been joined since, and all keep their order."""
+    require_gpu()
+    from paper_1606_02862_gb300 import pic, workloads as W
+
+    rng = np.random.default_rng(21)
+    N = 16
+    sc = (8, 4, 4)
+    x = rng.random((1500, 3)) * N
+    u = np.zeros_like(x)
+    v = 0.2 / W.DT_HALF_COURANT
+    x[:60, 1] = 4.0 * rng.integers(1, 4, 60) - 0.3  # past the face in the second step
+    u[:60, 1] = v / np.sqrt(1.0 - v * v)
+    box = W.BoxInit(N, N, N, particles=[(x, u, np.full(1500, 1e-12))])
+    wl = W.Workload("between", W.DT_HALF_COURANT, [W.SpeciesDef("e", -1.0, 1.0, shape)], [box])
+    ctx = ctx_from(wl, sc=sc, threads_per_sc=256, sort_every=4)
+
+    def lists():
+        p = ctx.read_particles(0, 0, ids=True)
+        home = np.floor(p["x"] / np.array(sc)).astype(int)
+        g = home[:, 0] + 2 * (home[:, 1] + 4 * home[:, 2])
+        node = np.floor(p["x"] + (0.5 if shape == 2 else 0.0)).astype(int) - home * np.array(sc)
+        return p["id"], g, node[:, 0] + 9 * (node[:, 1] + 5 * node[:, 2])
+
+    try:
+        ctx.step(3)
+        if shift:
+            ctx.shift_window(0, 4)
+        _, g, key = lists()
+        assert any(np.any(np.diff(key[g == k]) < 0) for k in range(32))  # arrivals at the lists' ends
+        ctx.step(1)
+        ids, g, key = lists()
+        assert np.all(np.diff(g) >= 0)  # read back list after list
+        for k in range(32):
+            assert np.all(np.diff(key[g == k]) >= 0), k
+        ctx.step(4)
+        assert np.array_equal(lists()[0], ids)
+        assert ctx.info(pic.INFO_STEPS) == 8
+    finally:
+        ctx.close()
