@@ -7,8 +7,7 @@
 // maintenance writes) from a work counter, one item ahead, so boxes of any
 // size and occupancy share one launch.  Per supercell:
 //   1. stage the E and B tile (supercell + G guard cells below, G = 1 for
-//      CIC/TSC, 2 with PCS) from HBM into shared memory with 16-byte
-//      asynchronous copies;
+//      CIC/TSC, 2 with PCS) from HBM into shared memory with two tensor loads;
 //   2. zero a shared J tile of the same extent;
 //   3. every thread takes particles of the supercell's frame lists: gather
 //      E, B from shared memory (CIC 2x2x2 / TSC 3x3x3 / PCS 4x4x4 weights
@@ -41,8 +40,8 @@
 // The push writes a deposit record
 // per particle; the deposit then runs in a lane order whose neighbours are
 // several list positions apart (dep_log_stride), so one warp's atomics land on
-// different nodes.  The current of a chunk accumulates in fixed point (see
-// chunk_scale).  Two deposit paths, both exact forms of that formula:
+// different nodes.  The current of a list accumulates in fixed point (see
+// kTileTerms).  Two deposit paths, both exact forms of that formula:
 //   common: on every axis the move stays on one spline piece -- the old and
 //     the new position round to the same node (TSC) / stay in the same cell
 //     (CIC, PCS) -- so the union of the two supports is 3 (TSC) / 2 (CIC) /
@@ -56,7 +55,7 @@
 //     whole groups of 32 lane-parallel, the leftover moves one per warp with
 //     all 32 lanes on the move's current lines.
 // The shared tiles use a row pitch of 4 mod 8 floats, so that rows are
-// 16-byte aligned (the E/B tile arrives by cp.async, the J tile leaves as
+// 16-byte aligned (the E/B tile arrives by tensor loads, the J tile leaves as
 // float4) and the 32 banks spread over neighbouring rows.
 #pragma once
 
@@ -424,30 +423,38 @@ __device__ __forceinline__ float esk_T(float s0e, float dse, float s0f, float ds
 
 // ------------------------------------------------------------ fixed-point J tile
 //
-// The shared J tile accumulates each chunk of particles in int32: shared-
-// memory int32 atomics are native, where FP32 shared atomics are a
-// compare-and-swap loop.  A chunk's contributions are scaled by a power of
-// two chosen from the chunk itself: with B = max over its particles and
-// axes of Tmax |jcoef_d w D_d| (|P| <= |D| and |T| <= Tmax = (max S)^2 bound
-// every term of the current by it) and n <= 256 particles, each scaled term is below 2^21 and a
-// node's sum below 2^30, so nothing overflows and a term keeps 2^-22 B
-// resolution.
-// After the chunk the integer tile is folded into an FP32 tile.  Scaled terms
-// convert to integers with the 1.5 * 2^23 magic-number add.
+// The shared J tile accumulates the current in int32: shared-memory int32
+// atomics are native, where FP32 shared atomics are a compare-and-swap loop.
+// Each chunk's contributions are scaled by a power of two chosen from the chunk
+// itself, so that every scaled term is below 2^kTermBits in magnitude: with B =
+// max over its particles and axes of Tmax |jcoef_d w D_d|, |P| <= |D| and |T| <=
+// Tmax = (max S)^2 bound every term of the current by B.  A particle adds one
+// term at most to a node's component, so a node's sum stays below 2^31 while
+// the tile holds at most kTileTerms particles at one scale: it is folded into
+// an FP32 tile before more come in and before a chunk of another scale (see
+// push_list).  A term keeps 2^-22 B resolution.  Scaled terms convert to
+// integers with the 1.5 * 2^23 magic-number add, which takes |x| < 2^22.
+constexpr int kTermBits = 21;
+constexpr int kTileTerms = 1023;
+// (the rounding of a term to an integer, 1/2 each, and the FP32 rounding of
+// the bound fit in the one term that is left)
+static_assert((long long)(kTileTerms + 1) << kTermBits <= 1LL << 31, "a node's sum fits in int32");
+static_assert(kTermBits < 22, "the magic-number range");
+static_assert(kGenDefer <= kTileTerms, "the moves set aside are folded once");
+
 __device__ __forceinline__ int magic_int(float x)
 {
     return __float_as_int(x + 12582912.0f) - 0x4B400000;
 }
 
-// scale = 2^(21 - e) with bound < 2^e: a scaled term is below 2^21
-// (magic-number range) and n <= 512 of them below 2^30.  Bounds below 2^-105
-// take that scale, which is the largest finite one (their terms are far below
-// anything FP32 fields resolve).
+// scale = 2^(kTermBits - e) with bound < 2^e.  Bounds below 2^-105 take that
+// scale, which is the largest finite one (their terms are far below anything
+// FP32 fields resolve).
 __device__ __forceinline__ float chunk_scale(float bound, float* inv)
 {
     const int e = bound > 0.0f ? max((__float_as_int(bound) >> 23) - 126, -105) : 0;
-    *inv = __int_as_float((127 + e - 21) << 23);
-    return __int_as_float((127 + 21 - e) << 23);
+    *inv = __int_as_float((127 + e - kTermBits) << 23);
+    return __int_as_float((127 + kTermBits - e) << 23);
 }
 
 // One window line pair: the M - 1 terms P[i] T of two parallel lines (tile
@@ -1291,11 +1298,12 @@ __device__ __forceinline__ int push_list(const StepDev& d, const SpeciesDev& sp,
     const int ls = SORTS ? 2 : dep_log_stride(n, S);
     // the integer tile holds the current of tile_n particles (of the chunks
     // since the last fold) at the scale 1 / tile_inv: it goes on collecting while
-    // the chunks' scales (powers of two) agree and n terms below 2^21 fit (256
+    // the chunks' scales (powers of two) agree and kTileTerms are not passed (256
     // threads, TSC: 128^3 at 8 per cell 0.980 -> 0.968 ms, 256^3 8.37 -> 8.33;
     // 128 threads, two particles each, 1.525 -> 1.553 ms, so those fold every
     // chunk, as CIC does, whose rounding stays)
-    constexpr int kTileMax = SORTS || NT < 256 ? 0 : 1023;
+    constexpr int kTileMax = SORTS || NT < 256 ? 0 : kTileTerms;
+    static_assert(C <= kTileTerms, "a chunk fits in the tile");
     float tile_inv = 0.0f;
     int tile_n = 0;
     int ndef = 0;  // general-window moves set aside in sh.gd
