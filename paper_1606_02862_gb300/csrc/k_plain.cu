@@ -7,6 +7,7 @@
 // supercell-sorted form is measured against.
 #include "pic_internal.cuh"
 #include "plain.cuh"
+#include "quotients.cuh"
 
 #include <cmath>
 
@@ -96,20 +97,6 @@ struct Axis64 {
             ni[k] = wrap(bi + k, n);
             nh[k] = wrap(bh + k, n);
         }
-    }
-};
-
-// Quotients n / g of one divisor, each rounded once: a step of Newton's on
-// n rg with the rounded reciprocal rg (Markstein 1990).  n rg alone moved the stored
-// positions of a few particles by a last bit, which shows in the displacements
-// of slow ones (1e-11 of the largest).  g beyond the largest double: 0, as n / g is.
-struct Over64 {
-    double g, rg;
-    __device__ __forceinline__ explicit Over64(double v) : g(v), rg(1.0 / v) {}
-    __device__ __forceinline__ double operator()(double n) const
-    {
-        const double q = n * rg;
-        return rg != 0.0 ? fma(fma(-q, g, n), rg, q) : q;
     }
 };
 

@@ -60,6 +60,7 @@
 #pragma once
 
 #include "pic_internal.cuh"
+#include "quotients.cuh"
 #include "tma.cuh"
 
 #include <cmath>
@@ -376,27 +377,6 @@ __device__ __forceinline__ void gather_pairs(const float* __restrict__ sF, int l
                                                 sF + 2 * N + (z.bh * TY + y.bi) * PX + x.bi, x.w, y.w, z.w);
     E[0] = BxEx.y, E[1] = EyBy.x, E[2] = BzEz.y;
     B[0] = BxEx.x, B[1] = EyBy.y, B[2] = BzEz.x;
-}
-
-// 1 / sqrt(x) for x >= 1 (rsqrtf without its care for denormals)
-__device__ __forceinline__ float rsqrt_ge1(float x)
-{
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// 2 / x for x >= 1: the approximate reciprocal and one step of Newton's
-// iteration for it, of x / 4, whose reciprocal is in FP32's normal range for
-// every finite x.  An x that overflowed gives 0, as the division does (Newton's
-// step alone would give 0 * infinity).
-__device__ __forceinline__ float two_over_ge1(float x)
-{
-    const float h = 0.25f * x;
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
-    r = fmaf(r, fmaf(-h, r, 1.0f), r);
-    return x == INFINITY ? 0.0f : 0.5f * r;
 }
 
 // Esirkepov's transverse factor S0e S0f + (DSe S0f + S0e DSf)/2 + DSe DSf / 3
