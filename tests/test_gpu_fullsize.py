@@ -2,7 +2,7 @@
 configuration the benchmark times: 256^3 periodic cells, 134,217,728 TSC
 electrons at 8 per cell (Maxwellian u_th = 0.05, density 0.01 on a fixed
 background), 8x4x4 supercells with 256 threads each, the step replayed
-from its CUDA graph, a sort pass every 4 steps.
+from its CUDA graph, the lists sorted every 4 steps.
 
 The oracle cannot step the whole box in seconds, so it steps windows of
 24^3 cells cut out of the GPU state (the fields and every particle inside),
@@ -11,14 +11,15 @@ it in one step: a TSC particle's gather and deposit windows reach 2.5 cells
 from it, the Yee update one cell per half step.  The comparison therefore
 keeps the cells and the particles at least 5 cells inside the window.
 One window straddles the periodic seam of the box on all three axes, where
-the deposit goes through the guard images.  The first step after the load
-(a sort pass of the push) and the next one (a stored-order pass) are both
-compared, on random E, B written over the whole box (the recipe itself
-starts from zero fields, which would leave the gather untested).
+the deposit goes through the guard images.  Three steps are compared: the
+first after the load (which sorts every list), the next one (stored order)
+and the fifth, which pushes the lists as the sort at the end of the fourth
+step left them.  All on random E, B written over the whole box (the recipe
+itself starts from zero fields, which would leave the gather untested).
 
 Then the 64^3 sub-run of the same recipe (2,097,152 particles, zero initial
-fields): the oracle follows the GPU from the load for 4 steps (one sort
-pass, three stored-order passes) and the state is compared at the end,
+fields): the oracle follows the GPU from the load for 4 steps, and for a
+fifth, whose lists the fourth one sorted; the state is compared after both,
 with the per-step tolerance times the number of steps.
 """
 import numpy as np
@@ -133,14 +134,22 @@ def test_headline_full_size_sampled_windows(orc):
         ctx.load_particles(0, 0, x, u, w)
         ctx.write_fields(0, pic.FIELD_E, E0)
         ctx.write_fields(0, pic.FIELD_B, B0)
-        # step 1: a sort pass, from the loaded state (ids are the load order)
+        # step 1: lists sorted after the load (ids are the load order)
         wins = _window_states(orc, W.DT_HALF_COURANT, E0, B0, x, u, w, np.arange(npart, dtype=np.int64))
         del x, u, w, E0, B0
         ctx.step(1)
         E1, B1, p1 = _step_and_compare(orc, ctx, wins, pic)
-        # step 2: a stored-order pass, from the GPU state after step 1
+        # step 2: stored order, from the GPU state after step 1
         wins = _window_states(orc, W.DT_HALF_COURANT, E1, B1, p1["x"], p1["u"], p1["w"], p1["id"])
         del E1, B1, p1
+        ctx.step(1)
+        _step_and_compare(orc, ctx, wins, pic)
+        # step 5: lists sorted at the end of step 4
+        ctx.step(2)
+        p = ctx.read_particles(0, 0, ids=True)
+        wins = _window_states(orc, W.DT_HALF_COURANT, ctx.read_fields(0, pic.FIELD_E), ctx.read_fields(0, pic.FIELD_B),
+                              p["x"], p["u"], p["w"], p["id"])
+        del p
         ctx.step(1)
         _step_and_compare(orc, ctx, wins, pic)
         assert ctx.count_particles(0, 0) == npart
@@ -162,5 +171,10 @@ def test_subrun_64_follows_the_oracle_for_four_steps(orc):
         tol = steps * TOL
         errs = compare_box(st, ids, ctx, wl, 0, tol_field=tol, tol_x=tol, tol_u=tol)
         print("64^3 sub-run errors after", steps, "steps:", errs)
+        ctx.step(1)
+        st.step(1)
+        tol = (steps + 1) * TOL
+        errs = compare_box(st, ids, ctx, wl, 0, tol_field=tol, tol_x=tol, tol_u=tol)
+        print("64^3 sub-run errors after", steps + 1, "steps:", errs)
     finally:
         ctx.close()

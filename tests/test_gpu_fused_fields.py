@@ -134,7 +134,7 @@ def test_fused_pair_against_the_oracle(orc):
     wl = _workload("uneven", seed=1)
     ctx = _ctx(wl, "uneven", pic.FIELD_UPDATE_FUSED)
     try:
-        ctx.step(1)  # a sort pass first, so that the pair has a stored-order pass
+        ctx.step(1)  # the pair pushes the lists in stored order, a step after their sort
         states = [oracle_state_from_gpu(orc, ctx, wl, b) for b in range(len(wl.boxes))]
         ctx.step(2)
         assert ctx.info(pic.INFO_FUSED_STEPS) == 2

@@ -49,8 +49,10 @@ def _thermal(n=(16, 16, 16), ppc=4, u_th=0.05, shape=2, seed=0, fields=1e-2, spe
 
 def _one_step_parity(orc, wl, tol, pre_steps=0, **ctx_kw):
     """pre_steps GPU steps first, then one compared step.  With the default
-    sort period of 4 the step after 0 pre-steps is a sort pass of the push
-    and the step after 1 to 3 pre-steps pushes the lists in stored order."""
+    sort period of 4: after 0 pre-steps TSC and PCS lists come from the sort
+    that follows a load and CIC lists are sorted in the push, 1 to 3 push the
+    lists in stored order, and after 4 TSC and PCS lists come from the sort at
+    the end of the fourth step and CIC lists are sorted in the push again."""
     require_gpu()
     ctx = ctx_from(wl, **ctx_kw)
     try:
@@ -79,7 +81,7 @@ def test_plain_fp64_one_step(orc, shape):
     _one_step_parity(orc, wl, PLAIN_TOL, precision=pic.PRECISION_FP64_PLAIN)
 
 
-@pytest.mark.parametrize("pre", [0, 2], ids=["sort_pass", "stored_order"])
+@pytest.mark.parametrize("pre", [0, 2, 4], ids=["after_load", "stored_order", "after_sort"])
 @pytest.mark.parametrize("shape", [1, 2])
 @pytest.mark.parametrize("sc,threads", [((4, 4, 4), 64), ((4, 4, 4), 128), ((8, 8, 4), 128),
                                         ((8, 8, 4), 256), ((8, 4, 4), 128), ((8, 4, 4), 256),
@@ -91,8 +93,8 @@ def test_mixed_one_step(orc, shape, sc, threads, pre):
 
 @pytest.mark.parametrize("sort_every", [1, 3])
 def test_mixed_sort_period(orc, sort_every):
-    """Every step a sort pass (1), or passes 1 and 2 in stored order after
-    a sort (3): the compared step is the one after two pre-steps."""
+    """A sort in every step (1), or two steps after the sort that follows the
+    load (3): the compared step is the one after two pre-steps."""
     wl = _thermal(n=(16, 16, 16), shape=2, u_th=0.1, species="ions")
     _one_step_parity(orc, wl, MIXED_TOL, pre_steps=2, sc=(8, 4, 4), threads_per_sc=256,
                      sort_every=sort_every)
@@ -209,7 +211,7 @@ def test_diagnostics_match_oracle(orc):
     ctx.close()
 
 
-@pytest.mark.parametrize("pre", [0, 2], ids=["sort_pass", "stored_order"])
+@pytest.mark.parametrize("pre", [0, 2, 4], ids=["after_load", "stored_order", "after_sort"])
 @pytest.mark.parametrize("shape", [1, 2])
 def test_mixed_energy_conserving_gather(orc, shape, pre):
     """The energy-conserving gather variant (one order lower along each
@@ -237,7 +239,7 @@ def test_plain_energy_conserving_gather(orc, shape):
 PCS_CONFIGS = [((4, 4, 4), 128), ((8, 4, 4), 256)]
 
 
-@pytest.mark.parametrize("pre", [0, 2], ids=["sort_pass", "stored_order"])
+@pytest.mark.parametrize("pre", [0, 2, 4], ids=["after_load", "stored_order", "after_sort"])
 @pytest.mark.parametrize("sc,threads", PCS_CONFIGS)
 def test_mixed_pcs_one_step(orc, sc, threads, pre):
     """The PCS (cubic spline) shape: 4-node gather, 4-node common and 5-node
