@@ -291,7 +291,10 @@ struct AxisPair {
             const float2 d = SWAP ? make_float2(dh, di) : make_float2(di, dh);
             const float2 a = __ffma2_rn(d, minus, half), c = __fadd2_rn(d, half);
             w[0] = __fmul2_rn(__fmul2_rn(half, a), a);
-            w[1] = __ffma2_rn(a, c, half);  // 3/4 - d^2
+            // 3/4 - d^2 within 4.5e-8 (rms 1.8e-8); as one fma of d within 3.0e-8
+            // (1.7e-8), which takes 0.3 % longer per step for the same error of
+            // the step
+            w[1] = __ffma2_rn(a, c, half);
             w[2] = __fmul2_rn(__fmul2_rn(half, c), c);
             if (ec) {
                 set_h(0, up ? 0.0f : 0.5f - o);
@@ -310,7 +313,9 @@ struct AxisPair {
             const float2 f2 = __fmul2_rn(f, f), g2 = __fmul2_rn(g, g);
             const float2 sixth = dup2(1.0f / 6.0f), two3 = dup2(2.0f / 3.0f);
             w[0] = __fmul2_rn(__fmul2_rn(g2, sixth), g);
-            w[1] = __ffma2_rn(f2, __ffma2_rn(half, f, minus), two3);  // (4 - 6 f^2 + 3 f^3) / 6
+            // (4 - 6 f^2 + 3 f^3) / 6 within 8.6e-8, f^3 / 6 within 3.7e-8 (9.1e-8 and
+            // 4.9e-8 with the sums of the definition times 1/6)
+            w[1] = __ffma2_rn(f2, __ffma2_rn(half, f, minus), two3);
             w[2] = __ffma2_rn(g2, __ffma2_rn(half, g, minus), two3);
             w[3] = __fmul2_rn(__fmul2_rn(f2, sixth), f);
             if (ec) {  // TSC at the half nodes cell-1, cell, cell+1
@@ -747,7 +752,7 @@ __device__ __forceinline__ void tsc_axis(TscAxis<V>& t, V di, V D, V c)
     const V half = vdup(0.5f, di), mhalf = vdup(-0.5f, di), third = vdup(1.0f / 3.0f, di);
     const V lo = vfma(di, vdup(-1.0f, di), half), hi = vadd(di, half);
     t.S0[0] = vmul(vmul(half, lo), lo);
-    t.S0[1] = vfma(lo, hi, half);  // 3/4 - di^2
+    t.S0[1] = vfma(lo, hi, half);  // 3/4 - di^2, as in AxisPair
     t.S0[2] = vmul(vmul(half, hi), hi);
     // DS = -D/2 (1 - d0 - d1), -D (d0 + d1), D/2 (1 + d0 + d1), d1 = d0 + D
     const V sum = vfma(vdup(2.0f, di), di, D);
